@@ -148,7 +148,7 @@ bool same_args(const SweepArgs &x, const SweepArgs &y) {
            x.surv_cap == y.surv_cap && x.cand == y.cand && x.stats == y.stats &&
            x.wave_children == y.wave_children && x.max_fan_shift == y.max_fan_shift && x.n_sys == y.n_sys &&
            x.single == y.single && x.blob_smem == y.blob_smem && x.tv_stride == y.tv_stride &&
-           x.eval_warps == y.eval_warps && x.rg.n == y.rg.n;
+           x.eval_warps == y.eval_warps && x.screen == y.screen && x.rg.n == y.rg.n;
 }
 
 // Builds a plan.  With `reuse` (a plan that is no longer needed) its stream, events,
@@ -318,6 +318,9 @@ int plan_create_impl(int32_t n_sys, const ivs_system *systems, const double *con
         if (d.shadow) max_tv = std::max(max_tv, d.n_tv);
     if (std::getenv("IVS_NO_COMBO")) max_tv = 0;   // per-child shadow evaluation instead of tables
     choose_eval_layout(a, max_tv);
+    a.screen = 0;
+    for (const DevSys &d : h.sys)
+        if (d.shadow && d.prefilter && d.j_poly >= 0 && !d.gap_split && (d.hs_enable || d.centred)) a.screen = 1;
     CUDA_TRY(configure_eval_kernels(a));
     CUDA_TRY(cudaMemcpyAsync(p->d_box_lo, roots_lo.data(), roots_lo.size() * 8, cudaMemcpyHostToDevice, p->stream));
     CUDA_TRY(cudaMemcpyAsync(p->d_box_hi, roots_hi.data(), roots_hi.size() * 8, cudaMemcpyHostToDevice, p->stream));

@@ -28,6 +28,7 @@
 #include "ivs_internal.h"
 #include "ivs_interval.cuh"
 #include "ivs_kernels.cuh"
+#include "ivs_screen.cuh"
 #include "ivs_tab.cuh"
 
 namespace ivs {
@@ -593,7 +594,7 @@ __device__ __forceinline__ void kr_block(double *sd, int *si, int t) {
 // boxes runs in the cooperative form, larger ones in the independent form (the other
 // kernel returns at once).
 template <int N, bool COOP>
-__device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int64_t coop_max) {
+__device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int64_t coop_max, int64_t screen_min) {
     using namespace hsd;
     using C = Cfg<N>;
     constexpr int BB = C::BB;
@@ -607,7 +608,9 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
     int *si = reinterpret_cast<int *>(sd + C::DOUBLES);
 
     WaveCtl *ctl = a.ctl;
-    const int64_t count = ctl->surv_count[N];
+    // the survivors, or the boxes that the FP32 screen left open when the sweep was screened
+    const bool screened = N >= kScreenMinVars && a.screen && ctl->surv_count[N] > screen_min;
+    const int64_t count = screened ? ctl->open_count[N] : ctl->surv_count[N];
     if (COOP ? count > coop_max : count <= coop_max) return;   // the other form's sweep
     int rank = 0, group = blockIdx.x;                         // group: this CTA or cluster
     if (COOP) {
@@ -620,7 +623,7 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
         copy_blob(smem, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);   // visible after the next barrier
     }
     const char *blob_smem = cache_blob ? smem : nullptr;
-    const Surv *list = a.surv + (size_t)N * a.surv_cap;
+    const Surv *list = screened ? a.cand + open_list_base(ctl, N) : a.surv + (size_t)N * a.surv_cap;
     const bool owner = t < BB;   // owner thread of box b = t
     for (int slot = 0;; slot ^= 1) {
         if (COOP) {
@@ -900,14 +903,14 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
 
 template <int N>
 __global__ void __launch_bounds__(hsd::Cfg<N>::NT, hsd::Cfg<N>::MIN_BLOCKS)
-    k_hs(SweepArgs a, int cache_blob, long long coop_max) {
-    hs_body<N, false>(a, cache_blob, coop_max);
+    k_hs(SweepArgs a, int cache_blob, long long coop_max, long long screen_min) {
+    hs_body<N, false>(a, cache_blob, coop_max, screen_min);
 }
 
 template <int N>
 __global__ void __cluster_dims__(hsd::kCS, 1, 1) __launch_bounds__(hsd::Cfg<N>::NT, 1)
-    k_hs_coop(SweepArgs a, int cache_blob, long long coop_max) {
-    hs_body<N, true>(a, cache_blob, coop_max);
+    k_hs_coop(SweepArgs a, int cache_blob, long long coop_max, long long screen_min) {
+    hs_body<N, true>(a, cache_blob, coop_max, screen_min);
 }
 
 // ---- launcher -------------------------------------------------------------------
@@ -916,6 +919,11 @@ __global__ void __cluster_dims__(hsd::kCS, 1, 1) __launch_bounds__(hsd::Cfg<N>::
 constexpr size_t kHsSmemLimit = 227 * 1024 - 64;
 // a cooperative CTA asks for at least this much, so no two share an SM
 constexpr size_t kOneCtaPerSm = 120 * 1024;
+
+// the screen's dynamic shared memory, less its static arrays
+constexpr size_t kScreenSmemLimit = 220 * 1024;
+// without the cooperative form (n > 12) a sweep of fewer boxes than this is not screened
+constexpr long long kScreenMin = 512;
 
 // resident clusters of the cooperative kernel for a shared memory size, queried once per
 // size (the launchers may run on several host threads)
@@ -928,24 +936,46 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     // cache the term table in shared memory when the plan holds one system and it fits
     const bool cache = a.single && (size_t)a.blob_smem + C::BYTES <= kHsSmemLimit;
     const size_t smem = (cache ? (size_t)a.blob_smem : 0) + C::BYTES;
-    long long coop_max = 0;
+    long long coop_max = 0, screen_min = kScreenMin;
+    int active_clusters = 0;
+    const size_t csmem = smem > kOneCtaPerSm ? smem : kOneCtaPerSm;
     if constexpr (N <= hsd::kCoopMaxN) {
       if (num_sms >= 2 * hsd::kCS) {
-        // narrow sweeps: clusters of kCS CTAs, one per SM, one chunk per cluster that can
-        // be resident at once (a wider sweep runs faster in the independent form)
-        const size_t csmem = smem > kOneCtaPerSm ? smem : kOneCtaPerSm;
         cudaError_t e = allow_max_dynamic_smem((const void *)k_hs_coop<N>);
         if (e != cudaSuccess) return e;
-        const int active_clusters = coop_clusters_cached((const void *)k_hs_coop<N>, num_sms, C::NT, csmem, &e);
+        active_clusters = coop_clusters_cached((const void *)k_hs_coop<N>, num_sms, C::NT, csmem, &e);
         if (e != cudaSuccess) return e;
         if (active_clusters > 0) {
             coop_max = (long long)active_clusters * C::BB;
-            k_hs_coop<N><<<active_clusters * hsd::kCS, C::NT, csmem, st>>>(a, cache ? 1 : 0, coop_max);
-            e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            *kernels = 2;
+            screen_min = coop_max;
         }
       }
+    }
+    if constexpr (N >= kScreenMinVars) {
+      if (a.screen) {
+        using S = scr::Cfg<N>;
+        const bool scache = a.single && (size_t)a.blob_smem + S::BYTES <= kScreenSmemLimit;
+        const size_t ssmem = (scache ? (size_t)a.blob_smem : 0) + S::BYTES;
+        cudaError_t e = allow_max_dynamic_smem((const void *)k_screen<N>);
+        if (e != cudaSuccess) return e;
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_screen<N>, S::NT, ssmem);
+        if (e != cudaSuccess) return e;
+        k_screen<N><<<num_sms * (per_sm < 1 ? 1 : per_sm), S::NT, ssmem, st>>>(a, scache ? 1 : 0, screen_min);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        ++*kernels;
+      }
+    }
+    if constexpr (N <= hsd::kCoopMaxN) {
+        if (active_clusters > 0) {
+            // narrow sweeps: clusters of kCS CTAs, one per SM, one chunk per cluster that can
+            // be resident at once (a wider sweep runs faster in the independent form)
+            k_hs_coop<N><<<active_clusters * hsd::kCS, C::NT, csmem, st>>>(a, cache ? 1 : 0, coop_max, screen_min);
+            cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+            ++*kernels;
+        }
     }
     cudaError_t e = allow_max_dynamic_smem((const void *)k_hs<N>);
     if (e != cudaSuccess) return e;
@@ -953,7 +983,7 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hs<N>, C::NT, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    k_hs<N><<<num_sms * per_sm, C::NT, smem, st>>>(a, cache ? 1 : 0, coop_max);
+    k_hs<N><<<num_sms * per_sm, C::NT, smem, st>>>(a, cache ? 1 : 0, coop_max, screen_min);
     return cudaGetLastError();
 }
 

@@ -126,6 +126,8 @@ struct WaveCtl {
     int32_t error;          // sticky: 1 = queue full
     int64_t surv_count[kMaxVars + 1];   // survivors per n (index n)
     int64_t hs_cursor[kMaxVars + 1];    // Hansen-Sengupta kernels' work cursors
+    int64_t screen_cursor[kMaxVars + 1];   // the FP32 screen's work cursors
+    int64_t open_count[kMaxVars + 1];      // boxes it left to the FP64 sweep
     int64_t cand_count;                 // FP32 survivors waiting for the FP64 evaluation
     int64_t cand_cursor;
     int64_t waves;

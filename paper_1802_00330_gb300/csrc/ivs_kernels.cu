@@ -50,6 +50,14 @@ constexpr size_t kBeginSmem = (size_t)kBeginThreads * kBeginPer;   // one byte p
 // with the sweep count.  Either way a region pops breadth first while under half full
 // and one parent at a time beyond; the schedule never changes a result.
 constexpr int kLasMax = 4096;
+__device__ __forceinline__ void reset_lists(WaveCtl *c) {
+    for (int n = 0; n <= kMaxVars; n++) {
+        c->surv_count[n] = 0;
+        c->hs_cursor[n] = 0;
+        c->screen_cursor[n] = 0;
+        c->open_count[n] = 0;
+    }
+}
 __device__ void wave_begin_regions(const SweepArgs &a, unsigned long long *s_key) {
     __shared__ long long s_red[kBeginThreads];
     __shared__ long long s_active, s_total, s_run;
@@ -170,7 +178,7 @@ __device__ void wave_begin_regions(const SweepArgs &a, unsigned long long *s_key
         c->children = kids;
         c->cursor = 0;
         c->staged = 0;
-        for (int n = 0; n <= kMaxVars; n++) { c->surv_count[n] = 0; c->hs_cursor[n] = 0; }
+        reset_lists(c);
         c->cand_count = 0;
         c->cand_cursor = 0;
         c->waves += 1;
@@ -225,7 +233,7 @@ __global__ void __launch_bounds__(kBeginThreads) k_wave_begin(SweepArgs a) {
         c->children = children;
         c->cursor = 0;
         c->staged = 0;
-        for (int n = 0; n <= kMaxVars; n++) { c->surv_count[n] = 0; c->hs_cursor[n] = 0; }
+        reset_lists(c);
         c->cand_count = 0;
         c->cand_cursor = 0;
         c->waves += 1;
@@ -286,7 +294,7 @@ __global__ void __launch_bounds__(kBeginThreads) k_wave_begin(SweepArgs a) {
     c->children = children;
     c->cursor = 0;
     c->staged = 0;
-    for (int n = 0; n <= kMaxVars; n++) { c->surv_count[n] = 0; c->hs_cursor[n] = 0; }
+    reset_lists(c);
     c->cand_count = 0;
     c->cand_cursor = 0;
     c->waves += 1;
@@ -346,7 +354,7 @@ __global__ void k_seed_roots(SweepArgs a, const double *box_lo, const double *bo
         c->cand_count = 0;
         c->cand_cursor = 0;
         c->wave_limit = 0x7FFFFFFFFFFFFFFFLL;
-        for (int n = 0; n <= kMaxVars; n++) { c->surv_count[n] = 0; c->hs_cursor[n] = 0; }
+        reset_lists(c);
     }
 }
 

@@ -36,6 +36,7 @@ struct SweepArgs {
     int32_t blob_smem;           // bytes of that blob
     int32_t tv_stride;           // term-combination entries per warp region (0: no tables)
     int32_t eval_warps;          // warps per block of k_eval
+    int32_t screen;              // 1: some system may be screened in FP32 (ivs_screen.cuh)
     DevRegions rg;               // serving: per-system queue regions (rg.n == 0: shared stack)
 };
 
@@ -74,7 +75,7 @@ cudaError_t launch_cancel_regions(const SweepArgs &a, const int32_t *d_cancel, c
 cudaError_t launch_admit(const SweepArgs &a, const double *d_lo, const double *d_hi, const int32_t *d_slot,
                          const int32_t *d_depth, int count, int n_max, cudaStream_t st);
 // Hansen-Sengupta + accept/split kernels for dimension n (ivs_hs_*.cu); *kernels receives
-// how many kernels the call launched (1, or 2 with the cooperative form)
+// how many kernels the call launched (1, or 2 with the cooperative form, one more with the screen)
 cudaError_t launch_hs_dim1(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels);
 cudaError_t launch_hs_dim2(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels);
 cudaError_t launch_hs_dim3(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels);
