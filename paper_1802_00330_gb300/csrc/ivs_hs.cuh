@@ -2,8 +2,8 @@
 // survived the evaluation (Section 2.3 eq 14, 17-22; Algorithm 3; Gauss-Jordan of
 // Section 2.4; Algorithm 4 products; Algorithm 1 termination (II); Algorithm 2 split).
 //
-// Mapping: one block takes BB boxes at a time (32; 16 for n >= 15) from an atomic
-// cursor, and its NW warps share the work of those boxes.  Lane b of every warp always
+// Mapping: one block takes BB boxes at a time (32; 16 for n >= 15; 8 in narrow sweeps,
+// below) from an atomic cursor, and its NW warps share the work of those boxes.  Lane b of every warp always
 // works on box b, so each FP64 warp instruction carries BB different boxes; the warps
 // split what is independent within a box: the n^2 + n polynomials of J(X) and f(x), the
 // row updates of each Gauss-Jordan step, the columns of M = B J(X), and the
@@ -18,11 +18,20 @@
 // Every value is computed by the same operations in the same order as the serial
 // definition, so the results are unchanged.  Matrices live in shared memory (structure
 // of arrays over the chunk's boxes: element (k, b) at k * BB + b, conflict-free).
+//
+// Narrow sweeps: a sweep whose boxes fit one round of 8-box chunks (k_hs_narrow) waits on
+// one chunk's dependent chain, not on the FP64 rate, so it takes small chunks on as many
+// SMs as there are and splits a box finer: the eliminations and M = B J(X) by single
+// entries.  A warp then carries 4 units of 8 boxes, so its FP64 instructions stay full; the
+// units of J(X) in one warp differ, which costs issue slots there but no time while few
+// blocks share an SM.  One chunk takes 30k cycles at n = 2, 65k at n = 5, 84k at n = 6, 120k
+// at n = 8, against 160-320k for a 32-box one.  (Clusters of 4 blocks that shared a 32-box
+// chunk through distributed shared memory, which this replaced, were slower: n = 2 25.6 ->
+// 23.7 us a sweep, n = 5 49.5 -> 44.4, the n = 6 solve's stage 0.80 -> 0.74 ms.)
 // Comparisons, sign tests, NaN and finiteness checks run on the integer pipes.
 // Templated on n; the instantiations are spread over several translation units
 // (ivs_hs_*.cu).
 #pragma once
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "ivs_internal.h"
@@ -33,12 +42,8 @@
 
 namespace ivs {
 
-namespace cg = cooperative_groups;
-
 namespace hsd {
 constexpr unsigned kFull = 0xFFFFFFFFu;
-constexpr int kCS = 4;          // CTAs per cluster in the cooperative form (8 measured no faster)
-constexpr int kCoopMaxN = 12;   // the cooperative form exists for n <= 12
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 __device__ __forceinline__ unsigned lanemask_lt() { return (1u << lane_id()) - 1u; }
 __device__ __forceinline__ unsigned long long *stat_ptr(const SweepArgs &a, int sys, int slot) {
@@ -67,9 +72,10 @@ __device__ __forceinline__ bool d_same(double a, double b) {
 }
 
 // Shared-memory layout of a block: arrays of rows, each row BB values (one per box).
-template <int N>
+template <int N, int B>
 struct Cfg {
-    static constexpr int BB = (N >= 15) ? 16 : 32;   // boxes per chunk
+    static constexpr int BB = B;                     // boxes per chunk
+    static constexpr bool NARROW = B < 16;           // units of single entries
     static constexpr int NW = (N <= 3) ? 4 : 8;      // warps per block
     static constexpr int NT = NW * 32;
     // blocks per SM: three for n = 7, 8 (80 registers, a few bytes of spill; measured 3-4%
@@ -122,23 +128,13 @@ struct ThinCol {
 // J(X) from the derivative polynomials compiled on the host (units q < N^2), and f(x)
 // at the midpoint x = mid X as a thin-box evaluation (units N^2 + i), for every box of
 // the chunk with I_JF set, by all threads of the block.
-// In the cooperative form (COOP) the cluster's CTAs share the units and every result is
-// written into each CTA's copy of the chunk (distributed shared memory); the barrier in
-// front keeps a fast CTA from overwriting J or f while a peer still reads the last pass's.
-template <int N, bool COOP>
+template <int N, int B>
 __device__ __forceinline__ void jf_block(const SweepArgs &a, const char *blob_smem, double *sd, const int *si,
                                          int t) {
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB, NT = C::NT;
     const int *jf = si + C::I_JF;
-    int gt = t, GT = NT;
-    if (COOP) {
-        cg::cluster_group cl = cg::this_cluster();
-        cl.sync();
-        gt = (int)cl.block_rank() * NT + t;
-        GT = kCS * NT;
-    }
-    for (int e = gt; e < (N * N + N) * BB; e += GT) {
+    for (int e = t; e < (N * N + N) * BB; e += NT) {
         const int q = e / BB, b = e % BB;
         if (!jf[b]) continue;
         const DevSys &S = a.tb.sys[si[C::I_SYS + b]];
@@ -153,39 +149,19 @@ __device__ __forceinline__ void jf_block(const SweepArgs &a, const char *blob_sm
             v = poly64(Tb, S.f_poly + i, ThinCol<BB>{sd + C::XC + b});
             dst = sd + C::FR + (2 * i) * BB + b;
         }
-        if (COOP) {
-            cg::cluster_group cl = cg::this_cluster();
-#pragma unroll
-            for (int r = 0; r < kCS; r++) {
-                double *d = cl.map_shared_rank(dst, r);
-                d[0] = v.lo;
-                d[BB] = v.hi;
-            }
-        } else {
-            dst[0] = v.lo;
-            dst[BB] = v.hi;
-        }
+        dst[0] = v.lo;
+        dst[BB] = v.hi;
     }
-    if (COOP) cg::this_cluster().sync();
-    else __syncthreads();
-}
-
-// rows per unit of the cooperative M = B J(X): the fewest that give every unit its own
-// warp of the cluster
-template <int N>
-__host__ __device__ constexpr int coop_rows() {
-    int r = 1;
-    while ((N + 1) * ((N + r - 1) / r) > kCS * Cfg<N>::NW) r++;
-    return r;
+    __syncthreads();
 }
 
 // Centred (mean-value) form from the expansion of Section 2.3 eq 13: for every y in X,
 // f_i(y) lies in F_c,i(X) = f_i(x) + sum_j J_ij(X) (X_j - x_j), folded left over
 // j = 1..n from f_i(x).  One equation per unit; sets I_CEX when some F_c,i excludes 0
 // (a NaN end never excludes).  Uses the J(X) and f(x) of jf_block.
-template <int N>
+template <int N, int B>
 __device__ __forceinline__ void centred_block(double *sd, int *si, int t) {
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB, NT = C::NT;
     const double *J = sd + C::JM;
     const int *cen = si + C::I_CEN;
@@ -210,9 +186,9 @@ __device__ __forceinline__ void centred_block(double *sd, int *si, int t) {
 // the sweep is skipped).
 // Parts: gj_block (mid J(X), Gauss-Jordan, column order), m_block (M = B J(X), r = B f(x)),
 // gs_block (Gauss-Seidel); each ends with a barrier.
-template <int N>
+template <int N, int B>
 __device__ __forceinline__ void gj_block(double *sd, int *si, int t) {
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB, NT = C::NT;
     double *J = sd + C::JM;   // interval (i, j): lo at (2 (i N + j)) BB, hi at (2 (i N + j) + 1) BB
     double *G = sd + C::GB;   // point (i, j) at (i N + j) BB
@@ -272,7 +248,27 @@ __device__ __forceinline__ void gj_block(double *sd, int *si, int t) {
             G[(k * N + j) * BB + b] = __ddiv_rn(j == k ? 1.0 : G[(k * N + j) * BB + b], pv);
         }
         __syncthreads();
-        // elimination of column k from the other rows (eq 24), one row per unit
+        // elimination of column k from the other rows (eq 24): one row per unit, or one
+        // entry per unit in narrow chunks (all read before any is written)
+        if constexpr (C::NARROW) {
+            constexpr int R = (N * N * BB + NT - 1) / NT;
+            double g[R];
+#pragma unroll
+            for (int q = 0; q < R; q++) {
+                const int e = t + q * NT, b = e % BB, j = e / BB % N, i = e / (BB * N);
+                g[q] = 0.0;
+                if (e >= N * N * BB || i == k || !run[b] || bad[b]) continue;
+                const double p = __dmul_rn(G[(i * N + k) * BB + b], G[(k * N + j) * BB + b]);
+                g[q] = __dsub_rn(j == k ? 0.0 : G[(i * N + j) * BB + b], p);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < R; q++) {
+                const int e = t + q * NT, b = e % BB, j = e / BB % N, i = e / (BB * N);
+                if (e >= N * N * BB || i == k || !run[b] || bad[b]) continue;
+                G[(i * N + j) * BB + b] = g[q];
+            }
+        } else
         for (int e = t; e < N * BB; e += NT) {
             const int i = e / BB, b = e % BB;
             if (i == k || !run[b] || bad[b]) continue;
@@ -314,48 +310,42 @@ __device__ __forceinline__ void gj_block(double *sd, int *si, int t) {
 
 // M = B J(X) in place of J, one column per unit; r = B f(x) in place of f (unit N)
 // (Algorithm 4, outward, u = 1..n in order; starting from the first product equals
-// starting from [0,0]).  Cooperative form: units are (column, block of coop_rows rows)
-// spread over the cluster, each holds its column in registers across a barrier before
-// any entry is overwritten, and writes its entries into every CTA's copy.
-template <int N, bool COOP>
+// starting from [0,0]).  Narrow chunks: one entry per unit, every entry formed before any
+// is overwritten.
+template <int N, int B>
 __device__ __forceinline__ void m_block(double *sd, const int *si, int t) {
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB, NT = C::NT;
     double *J = sd + C::JM;
     const double *G = sd + C::GB;
     const int *run = si + C::I_RUN;
     const int *bad = si + C::I_BAD;
-    if constexpr (COOP) {
-        constexpr int RB = coop_rows<N>(), NH = (N + RB - 1) / RB, U = (N + 1) * NH;
-        cg::cluster_group cl = cg::this_cluster();
-        const int gt = (int)cl.block_rank() * NT + t;
-        const int u = gt / BB, b = gt % BB;
-        const bool on = u < U && run[b] && !bad[b];
-        const int j = u / NH, h = u % NH;
-        ivd col[N];
-        if (on) {
+    if constexpr (C::NARROW) {
+        constexpr int R = ((N + 1) * N * BB + NT - 1) / NT;
+        ivd m[R];
 #pragma unroll
-            for (int v = 0; v < N; v++)
-                col[v] = (j < N) ? ivd{J[(2 * (v * N + j)) * BB + b], J[(2 * (v * N + j) + 1) * BB + b]}
-                                 : ivd{sd[C::FR + (2 * v) * BB + b], sd[C::FR + (2 * v + 1) * BB + b]};
+        for (int q = 0; q < R; q++) {
+            const int e = t + q * NT, b = e % BB, i = e / BB % N, j = e / (BB * N);
+            m[q] = ivd{0.0, 0.0};
+            if (e >= (N + 1) * N * BB || !run[b] || bad[b]) continue;
+            const double *c = (j < N) ? J + (2 * j) * BB + b : sd + C::FR + b;
+            const int step = (j < N) ? 2 * N * BB : 2 * BB;
+            ivd acc = iv_smul(G[(i * N) * BB + b], ivd{c[0], c[BB]});
+#pragma unroll
+            for (int u = 1; u < N; u++)
+                acc = iv_add(acc, iv_smul(G[(i * N + u) * BB + b], ivd{c[u * step], c[u * step + BB]}));
+            m[q] = acc;
         }
-        cl.sync();   // every column is read before any entry is overwritten
-        if (on) {
-            const int i1 = min(N, (h + 1) * RB);
-            for (int i = h * RB; i < i1; i++) {
-                ivd acc = iv_smul(G[(i * N) * BB + b], col[0]);
+        __syncthreads();
 #pragma unroll
-                for (int v = 1; v < N; v++) acc = iv_add(acc, iv_smul(G[(i * N + v) * BB + b], col[v]));
-                double *dst = (j < N) ? J + (2 * (i * N + j)) * BB + b : sd + C::FR + (2 * i) * BB + b;
-#pragma unroll
-                for (int r = 0; r < kCS; r++) {
-                    double *d = cl.map_shared_rank(dst, r);
-                    d[0] = acc.lo;
-                    d[BB] = acc.hi;
-                }
-            }
+        for (int q = 0; q < R; q++) {
+            const int e = t + q * NT, b = e % BB, i = e / BB % N, j = e / (BB * N);
+            if (e >= (N + 1) * N * BB || !run[b] || bad[b]) continue;
+            double *dst = (j < N) ? J + (2 * (i * N + j)) * BB + b : sd + C::FR + (2 * i) * BB + b;
+            dst[0] = m[q].lo;
+            dst[BB] = m[q].hi;
         }
-        cl.sync();
+        __syncthreads();
     } else {
     for (int e = t; e < (N + 1) * BB; e += NT) {
         const int j = e / BB, b = e % BB;
@@ -409,9 +399,9 @@ __device__ __forceinline__ void pair_sync() { asm volatile("bar.sync 1, 64;" :::
 // split) a row whose Y_i meets X_i in two pieces records its gap RN(lower end of the
 // upper piece - upper end of the lower piece) in gr when it is wider than the widest so
 // far; the row itself still takes the hull.
-template <int N>
+template <int N, int B>
 __device__ __forceinline__ void gs_block(double *sd, int *si, int t, GapRec &gr) {
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB, NT = C::NT, NP = N * (N - 1) / 2;
     static_assert(NT >= 128, "the rows need warps 0 and 1 and at least one more");
     double *J = sd + C::JM;
@@ -552,9 +542,9 @@ __device__ __forceinline__ void gs_block(double *sd, int *si, int t, GapRec &gr)
 // (X_j - x_j), folded over j = 1..n from the incoming box (rows are independent: one unit
 // per row and box), then Y_i = X_i intersected with K_i; a NaN leaves Y_i = X_i, an empty
 // intersection marks the box empty.  Runs after gs_block, which has set Y = X.
-template <int N>
+template <int N, int B>
 __device__ __forceinline__ void kr_block(double *sd, int *si, int t) {
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB, NT = C::NT;
     const double *J = sd + C::JM;
     const int *run = si + C::I_RUN;
@@ -586,22 +576,15 @@ __device__ __forceinline__ void kr_block(double *sd, int *si, int t) {
 }
 }  // namespace hsd
 
-// The kernel body.  Independent form (COOP = false): every CTA takes its own chunks.
-// Cooperative form (COOP = true, clusters of kCS CTAs, one CTA per SM): a cluster takes
-// a chunk and its CTAs work on it together -- each keeps a full copy of the chunk's state
-// and runs the serial parts itself (identical results on every copy), while J(X), f(x)
-// and M = B J(X) are shared out over the cluster's warps.  A sweep with at most coop_max
-// boxes runs in the cooperative form, larger ones in the independent form (the other
-// kernel returns at once).
-template <int N, bool COOP>
-__device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int64_t coop_max, int64_t screen_min) {
+// The kernel body.  A sweep with at most narrow_max boxes runs in narrow chunks, larger ones
+// in wide ones (the other kernel returns at once).
+template <int N, int B>
+__device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int64_t narrow_max, int64_t screen_min) {
     using namespace hsd;
-    using C = Cfg<N>;
+    using C = Cfg<N, B>;
     constexpr int BB = C::BB;
     extern __shared__ __align__(16) char smem[];
-    // chunk index, two slots used in turn: in the cooperative form the cluster's first CTA
-    // writes the next chunk's slot while a peer may not yet have read the current one
-    __shared__ long long s_base[2];
+    __shared__ long long s_base;   // first box of the chunk
     const int t = threadIdx.x, lane = (int)lane_id();
     const size_t blob_bytes = cache_blob ? (size_t)a.blob_smem : 0;
     double *sd = reinterpret_cast<double *>(smem + blob_bytes);
@@ -611,13 +594,8 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
     // the survivors, or the boxes that the FP32 screen left open when the sweep was screened
     const bool screened = N >= kScreenMinVars && a.screen && ctl->surv_count[N] > screen_min;
     const int64_t count = screened ? ctl->open_count[N] : ctl->surv_count[N];
-    if (COOP ? count > coop_max : count <= coop_max) return;   // the other form's sweep
-    int rank = 0, group = blockIdx.x;                         // group: this CTA or cluster
-    if (COOP) {
-        rank = (int)cg::this_cluster().block_rank();
-        group = blockIdx.x / kCS;
-    }
-    if ((int64_t)group * BB >= count) return;   // not needed for this many boxes (whole clusters)
+    if (C::NARROW ? count > narrow_max : count <= narrow_max) return;   // the other form's sweep
+    if ((int64_t)blockIdx.x * BB >= count) return;   // not needed for this many boxes
     if (cache_blob) {
         const DevSys &S0 = a.tb.sys[0];
         copy_blob(smem, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);   // visible after the next barrier
@@ -625,20 +603,10 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
     const char *blob_smem = cache_blob ? smem : nullptr;
     const Surv *list = screened ? a.cand + open_list_base(ctl, N) : a.surv + (size_t)N * a.surv_cap;
     const bool owner = t < BB;   // owner thread of box b = t
-    for (int slot = 0;; slot ^= 1) {
-        if (COOP) {
-            cg::cluster_group cl = cg::this_cluster();
-            if (rank == 0 && t == 0) {
-                const long long v = (long long)atomicAdd((unsigned long long *)&ctl->hs_cursor[N], (unsigned long long)BB);
-#pragma unroll
-                for (int r = 0; r < kCS; r++) *cl.map_shared_rank(&s_base[slot], r) = v;
-            }
-            cl.sync();
-        } else {
-            if (t == 0) s_base[slot] = (long long)atomicAdd((unsigned long long *)&ctl->hs_cursor[N], (unsigned long long)BB);
-            __syncthreads();
-        }
-        const long long base = s_base[slot];
+    for (;;) {
+        if (t == 0) s_base = (long long)atomicAdd((unsigned long long *)&ctl->hs_cursor[N], (unsigned long long)BB);
+        __syncthreads();
+        const long long base = s_base;
         if (base >= count) break;
         // the owners fetch their boxes: child `child` of queue entry `parent`
         bool active = false, stopped = false, dropped = false, dropped_c = false;
@@ -676,8 +644,7 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
             si[C::I_SYS + b] = sys;
             si[C::I_ITS + b] = its > cen ? its : cen;   // passes: the centred test needs J, f once
         }
-        // passes while some box wants one (a block-wide vote; in the cooperative form every
-        // CTA holds the same boxes, so all of them take the same number of passes)
+        // passes while some box wants one (a block-wide vote)
         const int my_passes = owner ? (its > cen ? its : cen) : 0;
         int my_cen = 0, my_kr = 0;   // this owner's box takes the centred test / Krawczyk step
         for (int it = 0; __syncthreads_or(my_passes > it); it++) {
@@ -697,15 +664,15 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
                 for (int k = 0; k < N; k++) si[C::I_ROWID + k * BB + b] = k;
             }
             __syncthreads();
-            jf_block<N, COOP>(a, blob_smem, sd, si, t);
-            if (__syncthreads_or(my_cen)) centred_block<N>(sd, si, t);
+            jf_block<N, B>(a, blob_smem, sd, si, t);
+            if (__syncthreads_or(my_cen)) centred_block<N, B>(sd, si, t);
             if (owner) {
                 const int b = t;
                 const bool run = si[C::I_HS + b] && !si[C::I_CEX + b];
                 si[C::I_RUN + b] = run ? (a.tb.sys[si[C::I_SYS + b]].krawczyk ? 2 : 1) : 0;
                 my_kr = si[C::I_RUN + b] == 2 ? 1 : 0;
                 st_app += run ? 1u : 0u;
-                if (run && it == 0 && rank == 0)   // every CTA of a cluster runs this; one counts
+                if (run && it == 0)
                     atomicAdd(stat_ptr(a, sys, ST_DEPTH_HS + (depth < kDepthSlots ? depth : kDepthSlots - 1)), 1ull);
                 if (si[C::I_CEX + b]) {
                     dropped_c = true;
@@ -718,10 +685,10 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
                 gr.w = 0.0;
             }
             __syncthreads();
-            gj_block<N>(sd, si, t);
-            m_block<N, COOP>(sd, si, t);
-            gs_block<N>(sd, si, t, gr);
-            if (__syncthreads_or(my_kr)) kr_block<N>(sd, si, t);
+            gj_block<N, B>(sd, si, t);
+            m_block<N, B>(sd, si, t);
+            gs_block<N, B>(sd, si, t, gr);
+            if (__syncthreads_or(my_kr)) kr_block<N, B>(sd, si, t);
             if (owner && si[C::I_RUN + t]) {
                 const int b = t;
                 if (si[C::I_EMPTY + b]) {
@@ -762,10 +729,9 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
             }
             __syncthreads();
         }
-        // Algorithm 1 termination (II) and the split, by warp 0 (lane b owns box b); in the
-        // cooperative form only the cluster's first CTA writes.  A box split at a gap takes
-        // a second pass with the upper piece in its gap coordinate.
-        if (t < 32 && rank == 0) {
+        // Algorithm 1 termination (II) and the split, by warp 0 (lane b owns box b).  A box
+        // split at a gap takes a second pass with the upper piece in its gap coordinate.
+        if (t < 32) {
             const int b = t;
             const int passes = __any_sync(kFull, two) ? 2 : 1;
             for (int pass = 0; pass < passes; pass++) {
@@ -898,92 +864,72 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
         }
         __syncthreads();   // the chunk's arrays and s_base are reused by the next chunk
     }
-    if (COOP) cg::this_cluster().sync();   // no CTA leaves while a peer may still write to it
 }
 
 template <int N>
-__global__ void __launch_bounds__(hsd::Cfg<N>::NT, hsd::Cfg<N>::MIN_BLOCKS)
-    k_hs(SweepArgs a, int cache_blob, long long coop_max, long long screen_min) {
-    hs_body<N, false>(a, cache_blob, coop_max, screen_min);
+constexpr int kWideBoxes = N >= 15 ? 16 : 32;
+constexpr int kNarrowBoxes = 8;
+
+template <int N>
+__global__ void __launch_bounds__(hsd::Cfg<N, kWideBoxes<N>>::NT, hsd::Cfg<N, kWideBoxes<N>>::MIN_BLOCKS)
+    k_hs(SweepArgs a, int cache_blob, long long narrow_max, long long screen_min) {
+    hs_body<N, kWideBoxes<N>>(a, cache_blob, narrow_max, screen_min);
 }
 
 template <int N>
-__global__ void __cluster_dims__(hsd::kCS, 1, 1) __launch_bounds__(hsd::Cfg<N>::NT, 1)
-    k_hs_coop(SweepArgs a, int cache_blob, long long coop_max, long long screen_min) {
-    hs_body<N, true>(a, cache_blob, coop_max, screen_min);
+__global__ void __launch_bounds__(hsd::Cfg<N, kNarrowBoxes>::NT, 2)
+    k_hs_narrow(SweepArgs a, int cache_blob, long long narrow_max, long long screen_min) {
+    hs_body<N, kNarrowBoxes>(a, cache_blob, narrow_max, screen_min);
 }
 
 // ---- launcher -------------------------------------------------------------------
 
 // largest dynamic shared memory a block may use (227 KB less the static s_base)
 constexpr size_t kHsSmemLimit = 227 * 1024 - 64;
-// a cooperative CTA asks for at least this much, so no two share an SM
-constexpr size_t kOneCtaPerSm = 120 * 1024;
-
 // the screen's dynamic shared memory, less its static arrays
 constexpr size_t kScreenSmemLimit = 220 * 1024;
-// without the cooperative form (n > 12) a sweep of fewer boxes than this is not screened
-constexpr long long kScreenMin = 512;
-
-// resident clusters of the cooperative kernel for a shared memory size, queried once per
-// size (the launchers may run on several host threads)
-int coop_clusters_cached(const void *func, int num_sms, int threads, size_t smem, cudaError_t *err);
 
 template <int N>
 static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels) {
-    *kernels = 1;
-    using C = hsd::Cfg<N>;
+    using C = hsd::Cfg<N, kWideBoxes<N>>;
+    using D = hsd::Cfg<N, kNarrowBoxes>;
+    *kernels = 2;
     // cache the term table in shared memory when the plan holds one system and it fits
     const bool cache = a.single && (size_t)a.blob_smem + C::BYTES <= kHsSmemLimit;
+    const bool ncache = a.single && (size_t)a.blob_smem + D::BYTES <= kHsSmemLimit;
     const size_t smem = (cache ? (size_t)a.blob_smem : 0) + C::BYTES;
-    long long coop_max = 0, screen_min = kScreenMin;
-    int active_clusters = 0;
-    const size_t csmem = smem > kOneCtaPerSm ? smem : kOneCtaPerSm;
-    if constexpr (N <= hsd::kCoopMaxN) {
-      if (num_sms >= 2 * hsd::kCS) {
-        cudaError_t e = allow_max_dynamic_smem((const void *)k_hs_coop<N>);
-        if (e != cudaSuccess) return e;
-        active_clusters = coop_clusters_cached((const void *)k_hs_coop<N>, num_sms, C::NT, csmem, &e);
-        if (e != cudaSuccess) return e;
-        if (active_clusters > 0) {
-            coop_max = (long long)active_clusters * C::BB;
-            screen_min = coop_max;
-        }
-      }
-    }
+    const size_t nsmem = (ncache ? (size_t)a.blob_smem : 0) + D::BYTES;
+    int per_sm = 0, n_per_sm = 0;   // blocks per SM at these shared memory sizes
+    cudaError_t e = allow_max_dynamic_smem((const void *)k_hs<N>);
+    if (e == cudaSuccess) e = allow_max_dynamic_smem((const void *)k_hs_narrow<N>);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hs<N>, C::NT, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n_per_sm, k_hs_narrow<N>, D::NT, nsmem);
+    if (e != cudaSuccess) return e;
+    if (per_sm < 1) per_sm = 1;
+    if (n_per_sm < 1) n_per_sm = 1;
+    // narrow sweeps: one round of narrow chunks
+    const long long narrow_max = (long long)num_sms * n_per_sm * D::BB;
+    const long long screen_min = narrow_max;
     if constexpr (N >= kScreenMinVars) {
       if (a.screen) {
         using S = scr::Cfg<N>;
         const bool scache = a.single && (size_t)a.blob_smem + S::BYTES <= kScreenSmemLimit;
         const size_t ssmem = (scache ? (size_t)a.blob_smem : 0) + S::BYTES;
-        cudaError_t e = allow_max_dynamic_smem((const void *)k_screen<N>);
+        e = allow_max_dynamic_smem((const void *)k_screen<N>);
         if (e != cudaSuccess) return e;
-        int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_screen<N>, S::NT, ssmem);
+        int s_per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s_per_sm, k_screen<N>, S::NT, ssmem);
         if (e != cudaSuccess) return e;
-        k_screen<N><<<num_sms * (per_sm < 1 ? 1 : per_sm), S::NT, ssmem, st>>>(a, scache ? 1 : 0, screen_min);
+        k_screen<N><<<num_sms * (s_per_sm < 1 ? 1 : s_per_sm), S::NT, ssmem, st>>>(a, scache ? 1 : 0, screen_min);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         ++*kernels;
       }
     }
-    if constexpr (N <= hsd::kCoopMaxN) {
-        if (active_clusters > 0) {
-            // narrow sweeps: clusters of kCS CTAs, one per SM, one chunk per cluster that can
-            // be resident at once (a wider sweep runs faster in the independent form)
-            k_hs_coop<N><<<active_clusters * hsd::kCS, C::NT, csmem, st>>>(a, cache ? 1 : 0, coop_max, screen_min);
-            cudaError_t e = cudaGetLastError();
-            if (e != cudaSuccess) return e;
-            ++*kernels;
-        }
-    }
-    cudaError_t e = allow_max_dynamic_smem((const void *)k_hs<N>);
+    k_hs_narrow<N><<<num_sms * n_per_sm, D::NT, nsmem, st>>>(a, ncache ? 1 : 0, narrow_max, screen_min);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    int per_sm = 0;   // blocks per SM at this shared memory size
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hs<N>, C::NT, smem);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    k_hs<N><<<num_sms * per_sm, C::NT, smem, st>>>(a, cache ? 1 : 0, coop_max, screen_min);
+    k_hs<N><<<num_sms * per_sm, C::NT, smem, st>>>(a, cache ? 1 : 0, narrow_max, screen_min);
     return cudaGetLastError();
 }
 

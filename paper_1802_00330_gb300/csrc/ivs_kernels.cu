@@ -8,8 +8,6 @@
 // roundings), so the sorted result set is identical to the serial solver's.
 #include <cuda_runtime.h>
 
-#include <mutex>
-
 #include "ivs_internal.h"
 #include "ivs_interval.cuh"
 #include "ivs_kernels.cuh"
@@ -764,39 +762,6 @@ static cudaError_t launch_hs(const SweepArgs &a, int n, int num_sms, cudaStream_
     case 16: return launch_hs_dim16(a, num_sms, st, kernels);
     default: return cudaErrorInvalidValue;
     }
-}
-
-// The answers live in a fixed table (no heap allocation, so the allocation-free entry
-// point may launch through here too); when it is full, further shapes are queried each
-// time instead of cached.
-int coop_clusters_cached(const void *func, int num_sms, int threads, size_t smem, cudaError_t *err) {
-    struct Known {
-        const void *func;
-        int num_sms, threads, dev, clusters;
-        size_t smem;
-    };
-    constexpr int kSlots = 512;
-    static std::mutex mu;
-    static Known known[kSlots];
-    static int used = 0;
-    int dev = 0;
-    *err = cudaGetDevice(&dev);
-    if (*err != cudaSuccess) return 0;
-    std::lock_guard<std::mutex> lk(mu);
-    for (int i = 0; i < used; i++) {
-        const Known &k = known[i];
-        if (k.func == func && k.num_sms == num_sms && k.threads == threads && k.smem == smem && k.dev == dev)
-            return k.clusters;
-    }
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)((num_sms / 4) * 4));
-    lc.blockDim = dim3((unsigned)threads);
-    lc.dynamicSmemBytes = smem;
-    int nc = 0;
-    *err = cudaOccupancyMaxActiveClusters(&nc, func, &lc);
-    if (*err != cudaSuccess) return 0;
-    if (used < kSlots) known[used++] = Known{func, num_sms, threads, dev, nc, smem};
-    return nc;
 }
 
 size_t eval_smem_bytes(const SweepArgs &a) {

@@ -7,8 +7,9 @@
 //                   c is set); optional FP32 outward evaluation, then FP64 evaluation
 //                   (Definition 1-2); survivors compacted with a warp ballot into a list
 //                   per dimension n
-//   k_hs<N>       : 32 survivors per block (narrow sweeps: per cluster of 4 blocks,
-//   k_hs_coop<N>    k_hs_coop): Hansen-Sengupta sweeps (Algorithm 3) or Krawczyk steps
+//   k_screen<N>   : decides in FP32 what the contraction would drop or leave unchanged
+//   k_hs<N>       : 32 survivors per block (narrow sweeps: 8 per block,
+//   k_hs_narrow<N>  k_hs_narrow): Hansen-Sengupta sweeps (Algorithm 3) or Krawczyk steps
 //                   (eq 15-16), then accept (Algorithm 1 (II)) or write the box as a
 //                   new parent
 //   k_commit      : moves the new parents onto the queue where the popped ones were
@@ -75,7 +76,7 @@ cudaError_t launch_cancel_regions(const SweepArgs &a, const int32_t *d_cancel, c
 cudaError_t launch_admit(const SweepArgs &a, const double *d_lo, const double *d_hi, const int32_t *d_slot,
                          const int32_t *d_depth, int count, int n_max, cudaStream_t st);
 // Hansen-Sengupta + accept/split kernels for dimension n (ivs_hs_*.cu); *kernels receives
-// how many kernels the call launched (1, or 2 with the cooperative form, one more with the screen)
+// how many kernels the call launched (2, one more with the screen)
 cudaError_t launch_hs_dim1(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels);
 cudaError_t launch_hs_dim2(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels);
 cudaError_t launch_hs_dim3(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels);

@@ -245,8 +245,8 @@ __device__ __forceinline__ long long open_list_base(const WaveCtl *c, int n) {
     return b;
 }
 
-// A sweep with at most `screen_min` boxes is not screened: it runs in one round of FP64
-// chunks, whose time is one chunk's latency whatever the number of boxes.
+// A sweep with at most `screen_min` boxes is not screened: it runs in one round of narrow
+// FP64 chunks, whose time is one chunk's latency whatever the number of boxes.
 template <int N>
 __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
     k_screen(SweepArgs a, int cache_blob, long long screen_min) {

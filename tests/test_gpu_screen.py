@@ -12,8 +12,8 @@ pytestmark = pytest.mark.gpu
 
 FATES = ("boxes", "hs_applied", "hs_empty", "hs_contracted", "hs_singular", "accepted", "unsplittable", "split",
          "max_depth_seen", "excluded_centred", "gap_splits", "depth_boxes", "depth_kept", "depth_hs")
-# a sweep is screened when it has more boxes than the cooperative form takes at once
-NARROW = 2048
+# a sweep is screened when it has more boxes than one round of narrow chunks takes
+NARROW = 152 * 2 * 8
 
 
 def _batched(n, seed):
@@ -61,7 +61,7 @@ def test_screened_equals_fp64_only(name):
     a = B.solve(s, **options)
     b = B.solve(s, prefilter_fp32=False, **options)
     assert a["status"] == b["status"]
-    assert int(np.max(a["stats"]["depth_hs"])) > (NARROW if s.n_vars <= 12 else 512) or name in ("n4", "n6_centred_alone", "n10_centred")
+    assert int(np.max(a["stats"]["depth_hs"])) > NARROW or name in ("n4", "n6_centred_alone", "n10_centred")
     for key in ("lo", "hi", "flags", "depth"):
         assert np.array_equal(a[key], b[key]), key
     for key in FATES:
