@@ -144,6 +144,7 @@ void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
     d.n_tv = E;
     d.n_cix = CX;
     d.blob_bytes = (int32_t)L.bytes;
+    d.head_bytes = (int32_t)L.head;
 }
 
 int validate(const ivs_system *s, const double *lo, const double *hi, const ivs_options *o) {

@@ -586,7 +586,7 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
     extern __shared__ __align__(16) char smem[];
     __shared__ long long s_base;   // first box of the chunk
     const int t = threadIdx.x, lane = (int)lane_id();
-    const size_t blob_bytes = cache_blob ? (size_t)a.blob_smem : 0;
+    const size_t blob_bytes = cache_blob ? (size_t)a.head_smem : 0;
     double *sd = reinterpret_cast<double *>(smem + blob_bytes);
     int *si = reinterpret_cast<int *>(sd + C::DOUBLES);
 
@@ -598,7 +598,7 @@ __device__ __forceinline__ void hs_body(const SweepArgs &a, int cache_blob, int6
     if ((int64_t)blockIdx.x * BB >= count) return;   // not needed for this many boxes
     if (cache_blob) {
         const DevSys &S0 = a.tb.sys[0];
-        copy_blob(smem, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);   // visible after the next barrier
+        copy_blob(smem, a.tb.blobs + S0.blob_off, (uint32_t)S0.head_bytes);   // visible after the next barrier
     }
     const char *blob_smem = cache_blob ? smem : nullptr;
     const Surv *list = screened ? a.cand + open_list_base(ctl, N) : a.surv + (size_t)N * a.surv_cap;
@@ -895,10 +895,10 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     using D = hsd::Cfg<N, kNarrowBoxes>;
     *kernels = 2;
     // cache the term table in shared memory when the plan holds one system and it fits
-    const bool cache = a.single && (size_t)a.blob_smem + C::BYTES <= kHsSmemLimit;
-    const bool ncache = a.single && (size_t)a.blob_smem + D::BYTES <= kHsSmemLimit;
-    const size_t smem = (cache ? (size_t)a.blob_smem : 0) + C::BYTES;
-    const size_t nsmem = (ncache ? (size_t)a.blob_smem : 0) + D::BYTES;
+    const bool cache = a.single && (size_t)a.head_smem + C::BYTES <= kHsSmemLimit;
+    const bool ncache = a.single && (size_t)a.head_smem + D::BYTES <= kHsSmemLimit;
+    const size_t smem = (cache ? (size_t)a.head_smem : 0) + C::BYTES;
+    const size_t nsmem = (ncache ? (size_t)a.head_smem : 0) + D::BYTES;
     int per_sm = 0, n_per_sm = 0;   // blocks per SM at these shared memory sizes
     cudaError_t e = allow_max_dynamic_smem((const void *)k_hs<N>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem((const void *)k_hs_narrow<N>);
@@ -913,8 +913,8 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     if constexpr (N >= kScreenMinVars) {
       if (a.screen) {
         using S = scr::Cfg<N>;
-        const bool scache = a.single && (size_t)a.blob_smem + S::BYTES <= kScreenSmemLimit;
-        const size_t ssmem = (scache ? (size_t)a.blob_smem : 0) + S::BYTES;
+        const bool scache = a.single && (size_t)a.head_smem + S::BYTES <= kScreenSmemLimit;
+        const size_t ssmem = (scache ? (size_t)a.head_smem : 0) + S::BYTES;
         e = allow_max_dynamic_smem((const void *)k_screen<N>);
         if (e != cudaSuccess) return e;
         int s_per_sm = 0;

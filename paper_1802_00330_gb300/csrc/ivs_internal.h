@@ -74,6 +74,7 @@ struct DevSys {
     int32_t n_cix;         // child-index entries (n_fterms << n; 0: none)
     int32_t krawczyk;      // 1: Krawczyk contraction (eq 15-16) instead of Gauss-Seidel
     int32_t bisect;        // 1: widest-coordinate bisection (2 children) instead of 2^n
+    int32_t head_bytes;    // bytes of the blob's head (ivs_tab.cuh)
     int32_t gap_split;     // 1: two boxes at an extended-division gap (Gauss-Seidel only)
 };
 

@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
     if ((int64_t)blockIdx.x * blockDim.x >= count) return;   // not needed for this many candidates
     if (a.single) {
         const DevSys &S0 = a.tb.sys[0];
-        copy_blob(s_blob, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);
+        copy_blob(s_blob, a.tb.blobs + S0.blob_off, (uint32_t)S0.head_bytes);
         __syncthreads();
     }
     const unsigned lane = lane_id();
@@ -795,13 +795,13 @@ static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int
                                      int use_cond, int *kernels) {
     int count = 4;   // wave_begin, eval, eval64, commit
     // ev (optional): n_hs_dims + 5 events recorded between the stages
-    const size_t blob = a.single ? (size_t)a.blob_smem : 0;
+    const size_t head = a.single ? (size_t)a.head_smem : 0;
     if (ev) cudaEventRecord(ev[0], st);
     k_wave_begin<<<1, kBeginThreads, kBeginSmem, st>>>(a);
     if (ev) cudaEventRecord(ev[1], st);
     k_eval<<<eval_blocks, a.eval_warps * 32, eval_smem_bytes(a), st>>>(a);
     if (ev) cudaEventRecord(ev[2], st);
-    k_eval64<<<num_sms * 4, kEval64Threads, blob, st>>>(a);
+    k_eval64<<<num_sms * 4, kEval64Threads, head, st>>>(a);
     if (ev) cudaEventRecord(ev[3], st);
     for (int q = 0; q < n_hs_dims; q++) {
         int kq = 0;

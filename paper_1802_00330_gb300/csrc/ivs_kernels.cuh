@@ -35,6 +35,7 @@ struct SweepArgs {
     int32_t n_sys;
     int32_t single;              // 1: one system; kernels cache its blob in shared memory
     int32_t blob_smem;           // bytes of that blob
+    int32_t head_smem;           // bytes of its head, all that the contraction's kernels cache
     int32_t tv_stride;           // term-combination entries per warp region (0: no tables)
     int32_t eval_warps;          // warps per block of k_eval
     int32_t screen;              // 1: some system may be screened in FP32 (ivs_screen.cuh)

@@ -131,6 +131,7 @@ bool pack_static(const ivs_system *s, DevSys &d) {
     d.n_fterms = 0;   // no per-parent combination table (the evaluation takes the direct path)
     d.n_tv = 0;
     d.blob_bytes = (int32_t)L.bytes;
+    d.head_bytes = (int32_t)L.head;
     return true;
 }
 
@@ -322,6 +323,7 @@ extern "C" int ivs_solve_noalloc(const ivs_system *s, const double *box_lo, cons
     a.n_sys = 1;
     a.single = 1;
     a.blob_smem = d.blob_bytes;
+    a.head_smem = d.head_bytes;
 
     // ---- upload (pageable copies from static host buffers; no allocation) ----
     const int32_t rd = o->root_depth;

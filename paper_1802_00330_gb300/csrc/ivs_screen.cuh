@@ -264,9 +264,9 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (cache_blob) {
         const DevSys &S0 = a.tb.sys[0];
-        copy_blob(smem, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);   // visible after the next barrier
+        copy_blob(smem, a.tb.blobs + S0.blob_off, (uint32_t)S0.head_bytes);   // visible after the next barrier
     }
-    float *sf = reinterpret_cast<float *>(smem + (cache_blob ? (size_t)a.blob_smem : 0));
+    float *sf = reinterpret_cast<float *>(smem + (cache_blob ? (size_t)a.head_smem : 0));
     double *sw = reinterpret_cast<double *>(reinterpret_cast<char *>(sf) + C::WOFF);
     const Surv *list = a.surv + (size_t)N * a.surv_cap;
     Surv *open = a.cand + open_list_base(ctl, N);

@@ -21,8 +21,11 @@ namespace ivs {
 // byte layout of a system blob with T terms, P polynomials, F factors, TF terms in the
 // equations F_i, E term-combination entries and CX child-index entries
 struct BlobLayout {
-    uint32_t cs, clo, chi, clo32, chi32, poly_off, tinfo, tv_off, tv_map, cix, fac, bytes;
+    uint32_t cs, clo, chi, clo32, chi32, poly_off, tinfo, fac, head, tv_off, tv_map, cix, bytes;
 };
+// The head (all that evaluates polynomials) comes first: kernels that do not read the
+// per-parent tables cache the head alone (at n = 8 5 KB of 45, a third block per SM for k_hs<8>
+// and k_screen<8> in plans of one system).
 __host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 0, int E = 0, int CX = 0) {
     BlobLayout L;
     uint32_t o = 0;
@@ -33,10 +36,12 @@ __host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 
     L.chi32 = o;     o += 4u * T;
     L.poly_off = o;  o += 4u * (P + 1);
     L.tinfo = o;     o += 4u * T;
+    L.fac = o;       o += (uint32_t)F;
+    o = (o + 15u) & ~15u;
+    L.head = o;
     L.tv_off = o;    o += 4u * (TF + 1);
     L.tv_map = o;    o += 4u * E;
     L.cix = o;       o += (2u * CX + 3u) & ~3u;
-    L.fac = o;       o += (uint32_t)F;
     L.bytes = (o + 15u) & ~15u;
     return L;
 }
