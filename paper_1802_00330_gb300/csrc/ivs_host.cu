@@ -147,8 +147,8 @@ bool same_args(const SweepArgs &x, const SweepArgs &y) {
            x.out.depth == y.out.depth && x.out.cap == y.out.cap && x.ctl == y.ctl && x.surv == y.surv &&
            x.surv_cap == y.surv_cap && x.cand == y.cand && x.stats == y.stats &&
            x.wave_children == y.wave_children && x.max_fan_shift == y.max_fan_shift && x.n_sys == y.n_sys &&
-           x.single == y.single && x.blob_smem == y.blob_smem && x.head_smem == y.head_smem && x.tv_stride == y.tv_stride &&
-           x.eval_warps == y.eval_warps && x.screen == y.screen && x.rg.n == y.rg.n;
+           x.single == y.single && x.blob_smem == y.blob_smem && x.head_smem == y.head_smem && x.tv_entries == y.tv_entries &&
+           x.eval_forms == y.eval_forms && x.screen == y.screen && x.rg.n == y.rg.n;
 }
 
 // Builds a plan.  With `reuse` (a plan that is no longer needed) its stream, events,
@@ -314,11 +314,11 @@ int plan_create_impl(int32_t n_sys, const ivs_system *systems, const double *con
     a.single = (n_sys == 1 && h.sys[0].blob_bytes <= 48 * 1024) ? 1 : 0;
     a.blob_smem = a.single ? h.sys[0].blob_bytes : 0;
     a.head_smem = a.single ? h.sys[0].head_bytes : 0;
-    int max_tv = 0;
-    for (const DevSys &d : h.sys)
-        if (d.shadow) max_tv = std::max(max_tv, d.n_tv);
-    if (std::getenv("IVS_NO_COMBO")) max_tv = 0;   // per-child shadow evaluation instead of tables
-    choose_eval_layout(a, max_tv);
+    choose_eval_layout(a, h.sys.data(), n_sys);
+    if (std::getenv("IVS_NO_COMBO")) {   // per-child evaluation instead of tables
+        a.tv_entries = 0;
+        a.eval_forms = 3;
+    }
     a.screen = 0;
     for (const DevSys &d : h.sys)
         if (d.shadow && d.prefilter && d.j_poly >= 0 && !d.gap_split && (d.hs_enable || d.centred)) a.screen = 1;

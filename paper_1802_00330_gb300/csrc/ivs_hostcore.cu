@@ -87,27 +87,39 @@ constexpr int kMaxTermCombos = 2048;
 
 void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
     const int T = (int)b.clo.size(), P = (int)b.poly_off.size() - 1, F = (int)b.fac.size();
-    std::vector<int32_t> tv_off{0};
+    // entries by the terms' number of factors and exponents, so that a warp that fills a
+    // table runs the same path on all lanes; a bisected parent has two children, which
+    // differ in its split coordinate alone: two entries a term
+    std::vector<int32_t> tv_off((size_t)n_fterms, 0);
     std::vector<uint32_t> tv_map;
+    std::vector<int> by_form((size_t)n_fterms);
+    for (int t = 0; t < n_fterms; t++) by_form[(size_t)t] = t;
+    auto form = [&](int t) {
+        std::vector<uint8_t> f{(uint8_t)term_nf(b.tinfo[t])};
+        for (int q = 0; q < term_nf(b.tinfo[t]); q++) f.push_back(b.fac[term_f0(b.tinfo[t]) + q] & 15u);
+        return f;
+    };
+    std::stable_sort(by_form.begin(), by_form.end(), [&](int x, int y) { return form(x) < form(y); });
     bool tv_ok = true;
-    for (int t = 0; t < n_fterms && tv_ok; t++) {
-        const int nf = term_nf(b.tinfo[t]);
-        if (nf > 8 || tv_off.back() + (1 << nf) > kMaxTermCombos) { tv_ok = false; break; }
-        for (int q = 0; q < (1 << nf); q++) tv_map.push_back(((uint32_t)t << 8) | (uint32_t)q);
-        tv_off.push_back(tv_off.back() + (1 << nf));
+    for (int t : by_form) {
+        const int nf = term_nf(b.tinfo[t]), combos = d.bisect ? 2 : 1 << nf;
+        if (nf > 8 || (int)tv_map.size() + combos > kMaxTermCombos) { tv_ok = false; break; }
+        tv_off[(size_t)t] = (int32_t)tv_map.size();
+        for (int q = 0; q < combos; q++) tv_map.push_back(((uint32_t)t << 8) | (uint32_t)q);
     }
     const int TF = tv_ok ? n_fterms : 0, E = tv_ok ? (int)tv_map.size() : 0;
-    // child-index table: for each F term and each child c (n bits), its table entry
-    // tv_off[t] + (c's bits in the term's variables); kept small (n <= 8, <= 16384 entries)
-    std::vector<uint16_t> cix;
-    if (TF > 0 && d.n <= 8 && (int64_t)TF << d.n <= 16384) {
-        cix.resize((size_t)TF << d.n);
+    // child-index table: for each F term, the combination bits of each pattern of the
+    // child's first 8 bits; kept small (64 KB)
+    std::vector<uint8_t> cix;
+    const int lb = std::min(d.n, 8);
+    if (TF > 0 && !d.bisect && ((int64_t)TF << lb) <= 65536) {
+        cix.resize((size_t)TF << lb);
         for (int t = 0; t < TF; t++) {
             const int nf = term_nf(b.tinfo[t]), f0 = term_f0(b.tinfo[t]);
-            for (int c = 0; c < (1 << d.n); c++) {
+            for (int c = 0; c < (1 << lb); c++) {
                 unsigned q = 0;
                 for (int f = 0; f < nf; f++) q |= ((unsigned)(c >> (b.fac[f0 + f] >> 4)) & 1u) << f;
-                cix[((size_t)t << d.n) + c] = (uint16_t)(tv_off[t] + (int)q);
+                cix[((size_t)t << lb) + c] = (uint8_t)q;
             }
         }
     }
@@ -131,10 +143,10 @@ void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
     }
     std::memcpy(base + L.poly_off, b.poly_off.data(), 4u * (P + 1));
     if (TF) {
-        std::memcpy(base + L.tv_off, tv_off.data(), 4u * (TF + 1));
+        std::memcpy(base + L.tv_off, tv_off.data(), 4u * TF);
         std::memcpy(base + L.tv_map, tv_map.data(), 4u * E);
     }
-    if (CX) std::memcpy(base + L.cix, cix.data(), 2u * CX);
+    if (CX) std::memcpy(base + L.cix, cix.data(), (size_t)CX);
     if (F) std::memcpy(base + L.fac, b.fac.data(), (size_t)F);
     d.blob_off = (int64_t)off;
     d.n_terms = T;
@@ -245,6 +257,15 @@ void compile_system(HostTables &h, const ivs_system *s, const ivs_options *o) {
     d.krawczyk = o->krawczyk ? 1 : 0;
     d.bisect = o->split_mode == 1 ? 1 : 0;
     d.gap_split = o->gap_split ? 1 : 0;
+    d.eval_block = (!d.bisect && n >= 9) ? 1 : 0;
+    if (m <= kMaxVars) {
+        int order[kMaxVars];
+        for (int i = 0; i < m; i++) order[i] = i;
+        std::stable_sort(order, order + m, [&](int x, int y) {
+            return bld.poly_off[x + 1] - bld.poly_off[x] < bld.poly_off[y + 1] - bld.poly_off[y];
+        });
+        for (int i = 0; i < m; i++) d.eq_order[i] = (uint8_t)order[i];
+    }
     pack_blob(h, bld, d, bld.poly_off[m]);
     h.sys.push_back(d);
 }

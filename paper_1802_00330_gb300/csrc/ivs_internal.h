@@ -71,7 +71,9 @@ struct DevSys {
     int32_t n_fterms;      // terms of the equations F_i
     int32_t n_tv;          // term-combination entries (0: no per-parent table)
     int32_t centred;       // 1: centred-form exclusion test before Hansen-Sengupta
-    int32_t n_cix;         // child-index entries (n_fterms << n; 0: none)
+    int32_t n_cix;         // child-index entries (n_fterms << min(n, 8); 0: none)
+    int32_t eval_block;    // 1: a parent's children are worth a block (512 or more)
+    uint8_t eq_order[kMaxVars];   // equations by number of terms (when m <= kMaxVars)
     int32_t krawczyk;      // 1: Krawczyk contraction (eq 15-16) instead of Gauss-Seidel
     int32_t bisect;        // 1: widest-coordinate bisection (2 children) instead of 2^n
     int32_t head_bytes;    // bytes of the blob's head (ivs_tab.cuh)

@@ -302,15 +302,31 @@ __device__ __forceinline__ shv sh_mul(shv x, shv y, bool &poison) {
     const bool ss = xs && ys;
     const float2 l1 = enc_mul_signed(lxh ? x.hd : x.ld, lxh ? x.hu : x.lu, lxh ? sxh : sxl,
                                      lyh ? y.hd : y.ld, lyh ? y.hu : y.lu, lyh ? syh : syl);
-    const float2 l2 = enc_mul_signed(ss ? x.hd : (lxh ? x.hd : x.ld), ss ? x.hu : (lxh ? x.hu : x.lu),
-                                     ss ? sxh : (lxh ? sxh : sxl), ss ? y.ld : (lyh ? y.hd : y.ld),
-                                     ss ? y.lu : (lyh ? y.hu : y.lu), ss ? syl : (lyh ? syh : syl));
     const float2 h1 = enc_mul_signed(uxh ? x.hd : x.ld, uxh ? x.hu : x.lu, uxh ? sxh : sxl,
                                      uyh ? y.hd : y.ld, uyh ? y.hu : y.lu, uyh ? syh : syl);
-    const float2 h2 = enc_mul_signed(ss ? x.hd : (uxh ? x.hd : x.ld), ss ? x.hu : (uxh ? x.hu : x.lu),
-                                     ss ? sxh : (uxh ? sxh : sxl), ss ? y.hd : (uyh ? y.hd : y.ld),
-                                     ss ? y.hu : (uyh ? y.hu : y.lu), ss ? syh : (uyh ? syh : syl));
-    return {fminf(l1.x, l2.x), fminf(l1.y, l2.y), fmaxf(h1.x, h2.x), fmaxf(h1.y, h2.y)};
+    // the second pair only when some lane of the warp has both operands straddling 0 (for
+    // the other lanes it repeats the first pair); a box's halves meet at 0 on these grids, so
+    // it is rare
+    if (__any_sync(__activemask(), ss)) {
+        const float2 l2 = enc_mul_signed(ss ? x.hd : (lxh ? x.hd : x.ld), ss ? x.hu : (lxh ? x.hu : x.lu),
+                                         ss ? sxh : (lxh ? sxh : sxl), ss ? y.ld : (lyh ? y.hd : y.ld),
+                                         ss ? y.lu : (lyh ? y.hu : y.lu), ss ? syl : (lyh ? syh : syl));
+        const float2 h2 = enc_mul_signed(ss ? x.hd : (uxh ? x.hd : x.ld), ss ? x.hu : (uxh ? x.hu : x.lu),
+                                         ss ? sxh : (uxh ? sxh : sxl), ss ? y.hd : (uyh ? y.hd : y.ld),
+                                         ss ? y.hu : (uyh ? y.hu : y.lu), ss ? syh : (uyh ? syh : syl));
+        return {fminf(l1.x, l2.x), fminf(l1.y, l2.y), fmaxf(h1.x, h2.x), fmaxf(h1.y, h2.y)};
+    }
+    return {l1.x, l1.y, h1.x, h1.y};
+}
+
+// c times x for a float c: sh_mul of the point interval [c, c], one product per end
+__device__ __forceinline__ shv sh_scale(float c, shv x, bool &poison) {
+    const int cx = sh_class(x);
+    poison |= cx == 0;
+    const float lu = cx == 2 ? fminf(x.lu, 0.0f) : x.lu;   // the ends clamped to their known sign
+    const float hd = cx == 1 ? fmaxf(x.hd, 0.0f) : x.hd;
+    if (c < 0.0f) return {__fmul_rd(c, x.hu), __fmul_ru(c, hd), __fmul_rd(c, lu), __fmul_ru(c, x.ld)};
+    return {__fmul_rd(c, x.ld), __fmul_ru(c, lu), __fmul_rd(c, hd), __fmul_ru(c, x.hu)};
 }
 
 // x^k (k >= 1) by the power rule of iv_pow.  Even k: the class picks the chain operands

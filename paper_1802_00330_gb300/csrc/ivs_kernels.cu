@@ -424,15 +424,6 @@ struct ChildCoordShadow {
         return shv{e[2 * up][j], e[2 * up + 1][j], e[2 * up + 2][j], e[2 * up + 3][j]};
     }
 };
-// coordinate of factor f of a table entry: the half is bit f of the combination q
-struct ComboCoordShadow {
-    const float (*e)[kMaxVars];
-    unsigned q;
-    __device__ __forceinline__ shv operator()(unsigned j, int f) const {
-        const unsigned up = (q >> f) & 1u;
-        return shv{e[2 * up][j], e[2 * up + 1][j], e[2 * up + 2][j], e[2 * up + 3][j]};
-    }
-};
 // box held in shared memory, structure of arrays with the given stride
 struct BoxCoord {
     const double *X;
@@ -469,80 +460,252 @@ __device__ __forceinline__ void push_cand(const SweepArgs &a, WaveCtl *ctl, bool
     }
 }
 
-// Children c0 + k G + r (k < K) of parent pi per thread, decided K at a time from the
-// parent's table (decide_from_table_k), then appended to the survivor / candidate lists.
-template <int K>
-__device__ __forceinline__ void table_children(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
-                                               const float4 *tv, uint32_t meta, int64_t pi, int n, unsigned fan,
-                                               unsigned r, unsigned G, unsigned &cnt_pre, unsigned &cnt_sh) {
-    for (unsigned c0 = 0; c0 < fan; c0 += K * G) {
-        unsigned c[K];
-        bool want[K];
-        int d[K];
-#pragma unroll
-        for (int k = 0; k < K; k++) {
-            c[k] = child_bits(S, meta, c0 + k * G + r);
-            want[k] = c0 + k * G + r < fan;
-        }
-        decide_from_table_k<K>(T, S, tv, c, want, d);
-#pragma unroll
-        for (int k = 0; k < K; k++) {
-            const bool keep = want[k] && d[k] == 1, cand = want[k] && d[k] == 2;
-            cnt_pre += (want[k] && d[k] == 0) ? 1u : 0u;
-            cnt_sh += keep ? 1u : 0u;
-            push_surv(a, ctl, n, keep, Surv{(uint32_t)pi, c[k]});
-            push_cand(a, ctl, cand, Surv{(uint32_t)pi, c[k]});
+// ---- decisions from a parent's table -------------------------------------------------------
+// A term's value over a child depends only on the child's halves in the term's variables,
+// so a parent's children share a table of the terms' values (ivs_tab.cuh): FP32 shadows, or
+// FP64 intervals when the system has no FP32 stage.  Both take 16 bytes an entry and hold
+// exactly what the per-child evaluation computes for the term.
+
+// states of a child: bit 0 some equation excludes 0, bit 1 some equation is open (shadow)
+enum : unsigned { CH_OUT = 1u, CH_OPEN = 2u };
+
+// coordinate of factor f of a table entry: bit f of q is the half (the split coordinate's
+// half alone for a bisected parent, whose other coordinates are not split)
+struct ComboCoordShadow {
+    const float (*e)[kMaxVars];
+    unsigned q;
+    int only;
+    __device__ __forceinline__ shv operator()(unsigned j, int f) const {
+        const unsigned up = only < 0 ? (q >> f) & 1u : (j == (unsigned)only ? q : 0u);
+        return shv{e[2 * up][j], e[2 * up + 1][j], e[2 * up + 2][j], e[2 * up + 3][j]};
+    }
+};
+struct ComboCoord64 {
+    const double (*p)[kMaxVars];
+    unsigned q;
+    int only;
+    __device__ __forceinline__ ivd operator()(unsigned j, int f) const {
+        const unsigned up = only < 0 ? (q >> f) & 1u : (j == (unsigned)only ? q : 0u);
+        return ivd{p[up][j], p[up + 1][j]};
+    }
+};
+
+// entries r, r + G, ... of a parent's table
+__device__ __forceinline__ void fill_table(const SysTab &T, const DevSys &S, float4 *tv, const double (*sp)[kMaxVars],
+                                           const float (*se)[kMaxVars], int only, unsigned r, unsigned G) {
+    for (int e = (int)r; e < S.n_tv; e += (int)G) {
+        const uint32_t mp = T.tv_map[e];
+        if (S.prefilter) {
+            tv[e] = term_shadow(T, (int)(mp >> 8), ComboCoordShadow{se, mp & 255u, only});
+        } else {
+            const ivd v = term_combo64(T, (int)(mp >> 8), ComboCoord64{sp, mp & 255u, only});
+            reinterpret_cast<double2 *>(tv)[e] = make_double2(v.lo, v.hi);
         }
     }
 }
 
-// The children of one parent, evaluated by a group of threads: one warp (GROUP = 32) or
-// the whole block.  r = the thread's rank in the group, G = the group size; every
-// thread of the group runs this with the same pi.  Three forms: the FP32 shadow (decides
-// what FP64 would decide with certainty; the undecided rest go to k_eval64), the plain
-// FP32 prefilter (its survivors go to k_eval64), or FP64 only.
+// table entry of term t for the child with bits c: the variables below 8 through the
+// child-index table (one byte a child), the others from the factors (in variable order)
+__device__ __forceinline__ int high_bits(const SysTab &T, int t, unsigned c) {
+    const uint32_t info = T.tinfo[t];
+    const int f0 = term_f0(info);
+    unsigned q = 0;
+    for (int f = term_nf(info) - 1; f >= 0; f--) {
+        const unsigned v = T.fac[f0 + f] >> 4;
+        if (v < 8) break;
+        q |= ((c >> v) & 1u) << f;
+    }
+    return (int)q;
+}
+__device__ __forceinline__ int entry_of(const SysTab &T, const DevSys &S, int t, unsigned c, int only) {
+    if (only >= 0) return T.tv_off[t] + (int)((c >> only) & 1u);
+    if (S.n_cix > 0) {
+        const int lb = S.n < 8 ? S.n : 8;
+        return T.tv_off[t] + (int)T.cix[((unsigned)t << lb) + (c & ((1u << lb) - 1u))] + (S.n > 8 ? high_bits(T, t, c) : 0);
+    }
+    const uint32_t info = T.tinfo[t];
+    const int nf = term_nf(info), f0 = term_f0(info);
+    unsigned q = 0;
+    for (int f = 0; f < nf; f++) q |= ((c >> (T.fac[f0 + f] >> 4)) & 1u) << f;
+    return T.tv_off[t] + (int)q;
+}
+
+// the running sums of one equation over one child, shadow or FP64, and their verdict
+struct SumShadow {
+    shv a;
+    __device__ __forceinline__ void set(const float4 *tv, int e) {
+        const float4 v = tv[e];
+        a = shv{v.x, v.y, v.z, v.w};
+    }
+    __device__ __forceinline__ void add(const float4 *tv, int e) {
+        const float4 v = tv[e];
+        a = sh_add(a, shv{v.x, v.y, v.z, v.w});
+    }
+    __device__ __forceinline__ void zero() { a = shv{0.f, 0.f, 0.f, 0.f}; }
+    __device__ __forceinline__ unsigned state() const {
+        if (a.ld > 0.0f || a.hu < 0.0f) return CH_OUT;
+        return (a.lu <= 0.0f && a.hd >= 0.0f) ? 0u : CH_OPEN;   // NaN (a poisoned term) is open
+    }
+};
+struct Sum64 {
+    ivd a;
+    __device__ __forceinline__ void set(const float4 *tv, int e) {
+        const double2 v = reinterpret_cast<const double2 *>(tv)[e];
+        a = ivd{v.x, v.y};
+    }
+    __device__ __forceinline__ void add(const float4 *tv, int e) {
+        const double2 v = reinterpret_cast<const double2 *>(tv)[e];
+        a = iv_add(a, ivd{v.x, v.y});
+    }
+    __device__ __forceinline__ void zero() { a = ivd{0.0, 0.0}; }
+    __device__ __forceinline__ unsigned state() const { return d_pos(a.lo) || d_neg(a.hi) ? CH_OUT : 0u; }
+};
+
+// state of child c under equation i, from the table
+template <class Sum>
+__device__ __forceinline__ unsigned table_state(const SysTab &T, const DevSys &S, const float4 *tv, int i, unsigned c,
+                                                int only) {
+    const int t0 = T.poly_off[S.f_poly + i], t1 = T.poly_off[S.f_poly + i + 1];
+    Sum s;
+    s.zero();
+    for (int t = t0; t < t1; t++) {
+        const int e = entry_of(T, S, t, c, only);
+        if (t == t0) s.set(tv, e);
+        else s.add(tv, e);
+    }
+    return s.state();
+}
+// the same without a table
+__device__ __forceinline__ unsigned direct_state(const SysTab &T, const DevSys &S, const double (*sp)[kMaxVars],
+                                                 const float (*se)[kMaxVars], int i, unsigned c) {
+    if (S.prefilter) {
+        bool poison = false;
+        const shv F = poly_shadow(T, S.f_poly + i, ChildCoordShadow{se, c}, poison);
+        if (poison) return CH_OPEN;
+        return SumShadow{F}.state();
+    }
+    return Sum64{poly64(T, S.f_poly + i, ChildCoord64{sp, c})}.state();
+}
+
+// One round of a warp over the children still in (entries [b0, b0 + 32 K) of `m` in `list`;
+// the first equation takes entry q = child q): equation i decides K children per lane, K
+// independent chains, and the ones that stay are packed to the front of the list.
+template <class Sum, int K>
+__device__ __forceinline__ void list_round(const SysTab &T, const DevSys &S, const float4 *tv, uint16_t *list, unsigned c0,
+                                           int i, bool first, unsigned b0, unsigned m, unsigned &out, unsigned &n_out) {
+    const unsigned lane = lane_id();
+    const int lb = S.n < 8 ? S.n : 8;
+    unsigned ent[K];
+    bool act[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        const unsigned q = b0 + (unsigned)k * 32u + lane;
+        act[k] = q < m;
+        ent[k] = first ? (act[k] ? q : 0u) : (act[k] ? (unsigned)list[q] : 0u);
+    }
+    Sum s[K];
+#pragma unroll
+    for (int k = 0; k < K; k++) s[k].zero();
+    const int t0 = T.poly_off[S.f_poly + i], t1 = T.poly_off[S.f_poly + i + 1];
+    const unsigned low0 = c0 & ((1u << lb) - 1u);
+    for (int t = t0; t < t1; t++) {
+        const int off = T.tv_off[t] + (S.n > 8 ? high_bits(T, t, c0) : 0);
+        const uint8_t *row = T.cix + ((unsigned)t << lb) + low0;
+#pragma unroll
+        for (int k = 0; k < K; k++) {
+            const int e = off + (int)row[ent[k] & 255u];
+            if (t == t0) s[k].set(tv, e);
+            else s[k].add(tv, e);
+        }
+    }
+    __syncwarp();   // every entry of the round has been read before any is written
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        const unsigned st = s[k].state();
+        const bool stay = act[k] && !(st & CH_OUT);
+        n_out += act[k] && (st & CH_OUT) ? 1u : 0u;
+        const unsigned bal = __ballot_sync(kFull, stay);
+        if (stay) list[out + __popc(bal & lanemask_lt())] = (uint16_t)(ent[k] | ((st & CH_OPEN) ? 256u : 0u));
+        out += __popc(bal);
+    }
+    __syncwarp();
+}
+
+// Children [c0, c0 + m) (m <= 256, c0 a multiple of m) of parent pi by one warp.  Every
+// equation excludes a third to a half of what is left, so the equations run over a list
+// of the children still in, packed after each: at n = 8 about 22 rounds of 32 instead of the
+// 64 that a lane per child takes (a warp's 32 lanes hardly ever finish early together).
+// Equations with fewer terms come first: cheaper, and narrower.  The survivors leave with
+// one reservation of the survivor list instead of one per 32 children.  (Evaluation of the
+// n = 8 plan, 6.4e7 children: 3.47 -> 2.35 ms; kinema, n = 9, 6.5e8: 62 -> 37 ms; n = 11, 3.2e7:
+// 23 -> 2.8 ms, where a table per warp had left one block per SM and no child index; 64-system
+// batch 144 -> 82 ms; the FP64-only n = 6 plan, whose children had no table: 0.91 -> 0.39 ms.)
+template <class Sum>
+__device__ __forceinline__ void list_children(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
+                                              const uint8_t *order, const float4 *tv, uint16_t *list, int64_t pi, unsigned c0,
+                                              unsigned m, unsigned &n_out, unsigned &n_keep) {
+    for (int q = 0; q < S.m && m > 0; q++) {
+        const int i = S.m <= kMaxVars ? (int)order[q] : q;
+        unsigned out = 0;
+        for (unsigned b0 = 0; b0 < m;) {
+            if (m - b0 > 64) {
+                list_round<Sum, 4>(T, S, tv, list, c0, i, q == 0, b0, m, out, n_out);
+                b0 += 128;
+            } else if (m - b0 > 32) {
+                list_round<Sum, 2>(T, S, tv, list, c0, i, q == 0, b0, m, out, n_out);
+                b0 += 64;
+            } else {
+                list_round<Sum, 1>(T, S, tv, list, c0, i, q == 0, b0, m, out, n_out);
+                b0 += 32;
+            }
+        }
+        m = out;
+    }
+    for (unsigned b0 = 0; b0 < m; b0 += 32) {
+        const bool act = b0 + lane_id() < m;
+        const unsigned ent = act ? (unsigned)list[b0 + lane_id()] : 0u;
+        const Surv sv{(uint32_t)pi, c0 + (ent & 255u)};
+        const bool keep = act && !(ent & 256u);
+        n_keep += keep ? 1u : 0u;
+        push_surv(a, ctl, S.n, keep, sv);
+        push_cand(a, ctl, act && (ent & 256u), sv);
+    }
+    __syncwarp();
+}
+
+// counts of one warp's children, in per-lane parts
+struct EvalCount {
+    unsigned pre, ev, e64, keep;
+};
+__device__ __forceinline__ void add_counts(const SweepArgs &a, int sys, const EvalCount &c) {
+    const unsigned pre = __reduce_add_sync(kFull, c.pre), ev = __reduce_add_sync(kFull, c.ev);
+    const unsigned e64 = __reduce_add_sync(kFull, c.e64), keep = __reduce_add_sync(kFull, c.keep);
+    if (lane_id() == 0) {
+        if (pre) atomicAdd(stat_ptr(a, sys, ST_EXCL_PREFILTER), (unsigned long long)pre);
+        if (ev) atomicAdd(stat_ptr(a, sys, ST_EXCL_EVAL), (unsigned long long)ev);
+        if (e64) atomicAdd(stat_ptr(a, sys, ST_EVAL64), (unsigned long long)e64);
+        if (keep) atomicAdd(stat_ptr(a, sys, ST_KEEP_SHADOW), (unsigned long long)keep);
+    }
+}
+__device__ __forceinline__ void add_parents(const SweepArgs &a, int sys, int depth, unsigned parents,
+                                            unsigned long long boxes) {
+    if (lane_id() == 0 && parents) {
+        atomicAdd(stat_ptr(a, sys, ST_LIVE), ~(unsigned long long)parents + 1ull);
+        atomicAdd(stat_ptr(a, sys, ST_BOXES), boxes);
+        if (boxes) atomicMax(stat_ptr(a, sys, ST_MAX_DEPTH), (unsigned long long)depth);
+        if (boxes) atomicAdd(stat_ptr(a, sys, ST_DEPTH_BOXES + (depth < kDepthSlots ? depth : kDepthSlots - 1)), boxes);
+    }
+}
+
 template <bool BLOCK>
 __device__ __forceinline__ void group_sync() {
     if (BLOCK) __syncthreads();
     else __syncwarp();
 }
 
-template <bool BLOCK>
-__device__ __forceinline__ void eval_parent(const SweepArgs &a, WaveCtl *ctl, const char *s_blob, float4 *s_tv,
-                                            double (*sp)[kMaxVars], float (*sf)[kMaxVars], float (*se)[kMaxVars],
-                                            int *s_flag, int64_t pi, unsigned r, unsigned G) {
-    const unsigned lane = lane_id();
-    const int sys = a.q.sys[pi];
-    const uint32_t meta = a.q.meta[pi];
-    const DevSys S = a.tb.sys[sys];
-    const SysTab T = make_tab(a.single ? s_blob : a.tb.blobs + S.blob_off, S);
-    const bool root = (meta & kRootFlag) != 0;
-    const int depth = (int)(meta & kDepthMask) + (root ? 0 : 1);
-    // the parent leaves the queue; past the box budget its children are dropped (the
-    // decision of rank 0, shared by the group)
-    int over = 0;
-    if (r == 0) {
-        atomicAdd(stat_ptr(a, sys, ST_LIVE), ~0ull);
-        if (S.max_boxes > 0) {
-            const unsigned long long done = *(volatile unsigned long long *)stat_ptr(a, sys, ST_BOXES);
-            if ((long long)done >= S.max_boxes) {
-                atomicOr(stat_ptr(a, sys, ST_FLAGS), (unsigned long long)kFlagBudget);
-                over = 1;
-            }
-        }
-        if (BLOCK) *s_flag = over;
-    }
-    if (BLOCK) {
-        __syncthreads();
-        over = *s_flag;
-    } else {
-        over = __shfl_sync(kFull, over, 0);
-    }
-    if (over) {
-        if (BLOCK) __syncthreads();   // s_flag is rewritten for the next parent
-        return;
-    }
-    const int n = S.n;
+// The parent's coordinates into shared memory, by the first n threads of its group
+__device__ __forceinline__ void load_parent(const SweepArgs &a, int64_t pi, int n, double (*sp)[kMaxVars],
+                                            float (*sf)[kMaxVars], float (*se)[kMaxVars], unsigned r) {
     if ((int)r < n) {
         const double lo = a.q.lo[r * a.q.cap + pi];
         const double mid = a.q.mid[r * a.q.cap + pi];
@@ -564,114 +727,332 @@ __device__ __forceinline__ void eval_parent(const SweepArgs &a, WaveCtl *ctl, co
         se[4][r] = hid;
         se[5][r] = hiu;
     }
-    group_sync<BLOCK>();
-    const unsigned fan = (unsigned)fan_out(S, meta);
-    unsigned cnt_pre = 0, cnt_ev = 0, cnt_64 = 0, cnt_sh = 0;
-    // per-parent term-combination table: when the fan-out fills warps and it fits
-    const bool use_tv = S.prefilter && S.shadow && S.n_tv > 0 && S.n_tv <= a.tv_stride && fan >= 32;
-    if (use_tv) {
-        for (int e = (int)r; e < S.n_tv; e += (int)G) {
-            const uint32_t mp = T.tv_map[e];
-            s_tv[e] = term_shadow(T, (int)(mp >> 8), ComboCoordShadow{se, mp & 255u});
+}
+
+// Children of one parent spread over a group (a warp, or a block of 256 threads) by
+// (equation, child) pairs, `chunk` children at a time: for few children, or few parents,
+// where lanes would idle otherwise and a thread that takes a child's equations one after the
+// other waits on their chain (evaluation of an n = 5 bisection, 35 narrow sweeps: 34 -> 16.5 us
+// a sweep; of the n = 6 solve: 0.31 -> 0.25 ms).  state: chunk words.
+template <bool BLOCK>
+__device__ __forceinline__ void pair_children(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
+                                              const float4 *tv, bool use_tv, const double (*sp)[kMaxVars],
+                                              const float (*se)[kMaxVars], unsigned *state, unsigned chunk, uint32_t meta,
+                                              int64_t pi, unsigned fan, int only, unsigned r, unsigned G, EvalCount &cnt) {
+    for (unsigned c0 = 0; c0 < fan; c0 += chunk) {
+        const unsigned cn = fan - c0 < chunk ? fan - c0 : chunk;
+        for (unsigned q = r; q < cn; q += G) state[q] = 0u;
+        group_sync<BLOCK>();
+        const unsigned pairs = cn * (unsigned)S.m;
+        for (unsigned e = r; e < pairs; e += G) {
+            const unsigned q = e % cn;
+            const int i = (int)(e / cn);
+            const unsigned c = child_bits(S, meta, c0 + q);
+            const unsigned st = !use_tv ? direct_state(T, S, sp, se, i, c)
+                                : S.prefilter ? table_state<SumShadow>(T, S, tv, i, c, only)
+                                              : table_state<Sum64>(T, S, tv, i, c, only);
+            if (st) atomicOr(&state[q], st);
+        }
+        group_sync<BLOCK>();
+        for (unsigned q0 = 0; q0 < cn; q0 += G) {
+            const bool act = q0 + r < cn;
+            const unsigned st = act ? state[q0 + r] : CH_OUT;
+            const bool keep = act && st == 0u, open = act && st == CH_OPEN;
+            const Surv sv{(uint32_t)pi, child_bits(S, meta, c0 + q0 + r)};
+            if (S.prefilter) {
+                cnt.pre += act && (st & CH_OUT) ? 1u : 0u;
+                cnt.keep += keep ? 1u : 0u;
+            } else {
+                cnt.e64 += act ? 1u : 0u;
+                cnt.ev += act && (st & CH_OUT) ? 1u : 0u;
+            }
+            push_surv(a, ctl, S.n, keep, sv);
+            if (S.prefilter) push_cand(a, ctl, open, sv);
         }
         group_sync<BLOCK>();
     }
-    // K children per thread (c0 + k G + r, k < K) on the table path with a child-index
-    // table when the fan-out fills K rounds of the group: K independent chains
-    const bool cix_tab = use_tv && S.n_cix > 0;
-    if (cix_tab && fan >= 4 * G) {
-        table_children<4>(a, ctl, T, S, s_tv, meta, pi, n, fan, r, G, cnt_pre, cnt_sh);
-    } else if (cix_tab && fan >= 2 * G) {
-        table_children<2>(a, ctl, T, S, s_tv, meta, pi, n, fan, r, G, cnt_pre, cnt_sh);
+}
+
+// Up to 16 children of one parent by one warp: lane e takes pairs e, e + 32, ... of (equation,
+// child), always of child e mod fan (fan is a power of two), and the lanes of a child join
+// their states with shuffles.
+__device__ __forceinline__ void few_children(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
+                                             const float4 *tv, bool use_tv, const double (*sp)[kMaxVars],
+                                             const float (*se)[kMaxVars], uint32_t meta, int64_t pi, unsigned fan, int only,
+                                             EvalCount &cnt) {
+    const unsigned lane = lane_id(), q = lane & (fan - 1u), pairs = fan * (unsigned)S.m;
+    const unsigned c = child_bits(S, meta, q);
+    unsigned st = 0u;
+    for (unsigned e = lane; e < pairs; e += 32u) {
+        const int i = (int)(e / fan);
+        st |= !use_tv ? direct_state(T, S, sp, se, i, c)
+              : S.prefilter ? table_state<SumShadow>(T, S, tv, i, c, only)
+                            : table_state<Sum64>(T, S, tv, i, c, only);
+    }
+    __syncwarp();
+    for (unsigned o = fan; o < 32u; o <<= 1) st |= __shfl_xor_sync(kFull, st, (int)o);
+    const bool act = lane < fan, keep = act && st == 0u, open = act && st == CH_OPEN;
+    const Surv sv{(uint32_t)pi, c};
+    if (S.prefilter) {
+        cnt.pre += act && (st & CH_OUT) ? 1u : 0u;
+        cnt.keep += keep ? 1u : 0u;
     } else {
+        cnt.e64 += act ? 1u : 0u;
+        cnt.ev += act && (st & CH_OUT) ? 1u : 0u;
+    }
+    push_surv(a, ctl, S.n, keep, sv);
+    if (S.prefilter) push_cand(a, ctl, open, sv);
+}
+
+// Without the shadow (magnitudes that float may not hold): the plain FP32 prefilter, one
+// child per thread; its survivors go to k_eval64.
+__device__ __forceinline__ void plain_children(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
+                                               const float (*sf)[kMaxVars], uint32_t meta, int64_t pi, unsigned fan,
+                                               unsigned r, unsigned G, EvalCount &cnt) {
+    for (unsigned c0 = 0; c0 < fan; c0 += G) {
+        const bool active = c0 + r < fan;
+        const unsigned c = child_bits(S, meta, c0 + r);
+        const bool cand = active && keep32(T, S, ChildCoord32{sf, c});
+        cnt.pre += active && !cand ? 1u : 0u;
+        push_cand(a, ctl, cand, Surv{(uint32_t)pi, c});
+    }
+}
+
+// Past its box budget a system's children are dropped.
+__device__ __forceinline__ bool over_budget(const SweepArgs &a, int sys, const DevSys &S) {
+    if (S.max_boxes <= 0) return false;
+    const unsigned long long done = *(volatile unsigned long long *)stat_ptr(a, sys, ST_BOXES);
+    if ((long long)done < S.max_boxes) return false;
+    atomicOr(stat_ptr(a, sys, ST_FLAGS), (unsigned long long)kFlagBudget);
+    return true;
+}
+
+// Whether a parent of system S takes a block in wide sweeps: its table does not fit a
+// warp's share of the region, or a block's warps each get 64 of its children or more.
+__device__ __forceinline__ bool block_form(const SweepArgs &a, const DevSys &S) {
+    return S.eval_block || S.n_tv > a.tv_entries / kEvalWarps;
+}
+
+// Without a table (more combinations than a region holds), one child per thread.
+__device__ __forceinline__ void direct_children(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
+                                                const double (*sp)[kMaxVars], const float (*se)[kMaxVars], uint32_t meta,
+                                                int64_t pi, unsigned fan, unsigned r, unsigned G, EvalCount &cnt) {
     for (unsigned c0 = 0; c0 < fan; c0 += G) {
         const bool active = c0 + r < fan;
         const unsigned c = child_bits(S, meta, c0 + r);
         bool keep = false, cand = false;
-        if (active) {
-            if (use_tv) {
-                const int d = decide_from_table(T, S, s_tv, c);
-                keep = d == 1;
-                cand = d == 2;
-                cnt_pre += d == 0 ? 1u : 0u;
-                cnt_sh += keep ? 1u : 0u;
-            } else if (S.prefilter && S.shadow) {
-                const int d = decide_shadow(T, S, ChildCoordShadow{se, c});
-                keep = d == 1;
-                cand = d == 2;
-                cnt_pre += d == 0 ? 1u : 0u;
-                cnt_sh += keep ? 1u : 0u;
-            } else if (S.prefilter) {
-                cand = keep32(T, S, ChildCoord32{sf, c});
-                cnt_pre += cand ? 0u : 1u;
-            } else {
-                cnt_64 += 1;
-                keep = keep64(T, S, ChildCoord64{sp, c});
-                cnt_ev += keep ? 0u : 1u;
-            }
+        if (active && S.prefilter) {
+            const int d = decide_shadow(T, S, ChildCoordShadow{se, c});
+            keep = d == 1;
+            cand = d == 2;
+            cnt.pre += d == 0 ? 1u : 0u;
+            cnt.keep += keep ? 1u : 0u;
+        } else if (active) {
+            cnt.e64 += 1;
+            keep = keep64(T, S, ChildCoord64{sp, c});
+            cnt.ev += keep ? 0u : 1u;
         }
-        push_surv(a, ctl, n, keep, Surv{(uint32_t)pi, c});
-        push_cand(a, ctl, cand, Surv{(uint32_t)pi, c});
+        push_surv(a, ctl, S.n, keep, Surv{(uint32_t)pi, c});
+        if (S.prefilter) push_cand(a, ctl, cand, Surv{(uint32_t)pi, c});
     }
-    }
-    cnt_pre = __reduce_add_sync(kFull, cnt_pre);
-    cnt_ev = __reduce_add_sync(kFull, cnt_ev);
-    cnt_64 = __reduce_add_sync(kFull, cnt_64);
-    cnt_sh = __reduce_add_sync(kFull, cnt_sh);
-    if (lane == 0) {
-        if (r == 0) {
-            atomicAdd(stat_ptr(a, sys, ST_BOXES), (unsigned long long)fan);
-            atomicMax(stat_ptr(a, sys, ST_MAX_DEPTH), (unsigned long long)depth);
-            atomicAdd(stat_ptr(a, sys, ST_DEPTH_BOXES + (depth < kDepthSlots ? depth : kDepthSlots - 1)),
-                      (unsigned long long)fan);
-        }
-        if (cnt_pre) atomicAdd(stat_ptr(a, sys, ST_EXCL_PREFILTER), (unsigned long long)cnt_pre);
-        if (cnt_ev) atomicAdd(stat_ptr(a, sys, ST_EXCL_EVAL), (unsigned long long)cnt_ev);
-        if (cnt_64) atomicAdd(stat_ptr(a, sys, ST_EVAL64), (unsigned long long)cnt_64);
-        if (cnt_sh) atomicAdd(stat_ptr(a, sys, ST_KEEP_SHADOW), (unsigned long long)cnt_sh);
-    }
-    group_sync<BLOCK>();   // the parent's arrays are rewritten for the next parent
 }
 
-// Children of the popped parents.  A wide sweep gives each warp a parent at a time from
-// a shared cursor (one lane per child, or two or four children per lane on the table
-// path when the fan-out fills that many rounds); a narrow one (at most one parent per block)
-// gives each block its parents and spreads a parent's table entries and children over
-// all of the block's threads, so the few parents of the first and last sweeps finish
-// sooner.  Both run the same per-child arithmetic.
+// children [c0, c0 + m) by one warp through list_children, with the counts of either mode
+__device__ __forceinline__ void listed(const SweepArgs &a, WaveCtl *ctl, const SysTab &T, const DevSys &S,
+                                       const uint8_t *order, const float4 *tv, uint16_t *list, int64_t pi, unsigned c0,
+                                       unsigned m, EvalCount &cnt) {
+    unsigned n_out = 0, n_keep = 0;
+    if (S.prefilter) {
+        list_children<SumShadow>(a, ctl, T, S, order, tv, list, pi, c0, m, n_out, n_keep);
+        cnt.pre += n_out;
+        cnt.keep += n_keep;
+    } else {
+        list_children<Sum64>(a, ctl, T, S, order, tv, list, pi, c0, m, n_out, n_keep);
+        cnt.ev += n_out;
+        cnt.e64 += lane_id() == 0 ? m : 0u;
+    }
+}
+
+// What a warp has counted for the system and depth of its last parents: added to the
+// system's counters when either changes and at the end, not parent by parent (six atomics on
+// the same six addresses for each of the 16384 parents of an n = 8 sweep).
+struct WarpTally {
+    int sys, depth;
+    unsigned parents;
+    unsigned long long boxes;
+    EvalCount cnt;
+};
+__device__ __forceinline__ void flush_tally(const SweepArgs &a, WarpTally &w) {
+    if (w.parents) {
+        add_counts(a, w.sys, w.cnt);
+        add_parents(a, w.sys, w.depth, w.parents, w.boxes);
+    }
+    w.parents = 0;
+    w.boxes = 0;
+    w.cnt = EvalCount{0u, 0u, 0u, 0u};
+}
+
+// One parent per warp.
+__device__ __forceinline__ void eval_warp(const SweepArgs &a, WaveCtl *ctl, const char *s_blob, float4 *s_tv,
+                                          double (*sp)[kMaxVars], float (*sf)[kMaxVars], float (*se)[kMaxVars],
+                                          uint16_t *list, int64_t pi, WarpTally &w) {
+    const unsigned lane = lane_id();
+    const int sys = a.q.sys[pi];
+    const uint32_t meta = a.q.meta[pi];
+    const DevSys S = a.tb.sys[sys];
+    if (block_form(a, S)) return;   // the block pass takes it
+    const SysTab T = make_tab(a.single ? s_blob : a.tb.blobs + S.blob_off, S);
+    const bool root = (meta & kRootFlag) != 0;
+    const int depth = (int)(meta & kDepthMask) + (root ? 0 : 1);
+    if (sys != w.sys || depth != w.depth || S.max_boxes > 0) {
+        flush_tally(a, w);
+        w.sys = sys;
+        w.depth = depth;
+    }
+    w.parents += 1;
+    int over = 0;
+    if (lane == 0) over = over_budget(a, sys, S) ? 1 : 0;
+    if (__shfl_sync(kFull, over, 0)) return;
+    const unsigned fan = (unsigned)fan_out(S, meta);
+    w.boxes += fan;
+    load_parent(a, pi, S.n, sp, sf, se, lane);
+    __syncwarp();
+    const bool plain = S.prefilter && !S.shadow;
+    // a round of short equations is sooner evaluated than a table filled for it
+    const bool brief = fan * (unsigned)S.m <= 32u && S.n_fterms <= 4 * S.m;
+    const bool use_tv = !plain && !brief && S.n_tv > 0 && S.n_tv <= a.tv_entries / kEvalWarps;
+    const int only = S.bisect ? (int)((meta >> kSplitShift) & kSplitMask) : -1;
+    if (use_tv) {
+        fill_table(T, S, s_tv, sp, se, only, lane, 32u);
+        __syncwarp();
+    }
+    if (plain) {
+        plain_children(a, ctl, T, S, sf, meta, pi, fan, lane, 32u, w.cnt);
+    } else if (use_tv && fan >= 32 && S.n_cix > 0) {
+        for (unsigned c0 = 0; c0 < fan; c0 += 256)
+            listed(a, ctl, T, S, a.tb.sys[sys].eq_order, s_tv, list, pi, c0, fan - c0 < 256 ? fan - c0 : 256, w.cnt);
+    } else if (fan < 32) {
+        few_children(a, ctl, T, S, s_tv, use_tv, sp, se, meta, pi, fan, only, w.cnt);
+    } else if (use_tv) {
+        pair_children<false>(a, ctl, T, S, s_tv, use_tv, sp, se, reinterpret_cast<unsigned *>(list), 64u, meta, pi, fan, only,
+                             lane, 32u, w.cnt);
+    } else {
+        direct_children(a, ctl, T, S, sp, se, meta, pi, fan, lane, 32u, w.cnt);
+    }
+    __syncwarp();   // the parent's arrays are rewritten for the next parent
+}
+
+// One parent per block: its table is filled by all threads; many children go to the warps
+// in equal parts (list_children), few are spread by (equation, child) pairs.
+__device__ __forceinline__ void eval_block(const SweepArgs &a, WaveCtl *ctl, const char *s_blob, float4 *s_tv,
+                                           double (*sp)[kMaxVars], float (*sf)[kMaxVars], float (*se)[kMaxVars],
+                                           uint16_t *lists, int *s_flag, int64_t pi) {
+    const unsigned t = threadIdx.x, warp = t >> 5;
+    const int sys = a.q.sys[pi];
+    const uint32_t meta = a.q.meta[pi];
+    const DevSys S = a.tb.sys[sys];
+    const SysTab T = make_tab(a.single ? s_blob : a.tb.blobs + S.blob_off, S);
+    const bool root = (meta & kRootFlag) != 0;
+    const int depth = (int)(meta & kDepthMask) + (root ? 0 : 1);
+    if (t == 0) *s_flag = over_budget(a, sys, S) ? 1 : 0;
+    load_parent(a, pi, S.n, sp, sf, se, t);
+    __syncthreads();
+    const bool over = *s_flag != 0;
+    const unsigned fan = (unsigned)fan_out(S, meta);
+    if (!over) {
+        const bool plain = S.prefilter && !S.shadow;
+        const bool use_tv = !plain && S.n_tv > 0 && S.n_tv <= a.tv_entries;
+        const int only = S.bisect ? (int)((meta >> kSplitShift) & kSplitMask) : -1;
+        EvalCount cnt{0u, 0u, 0u, 0u};
+        if (use_tv) {
+            fill_table(T, S, s_tv, sp, se, only, t, kEvalThreads);
+            __syncthreads();
+        }
+        if (plain) {
+            plain_children(a, ctl, T, S, sf, meta, pi, fan, t, kEvalThreads, cnt);
+        } else if (use_tv && fan >= 512 && S.n_cix > 0) {
+            const unsigned m = fan / kEvalWarps < 256 ? fan / kEvalWarps : 256;
+            for (unsigned c0 = warp * m; c0 < fan; c0 += kEvalWarps * m)
+                listed(a, ctl, T, S, a.tb.sys[sys].eq_order, s_tv, lists + warp * 256, pi, c0, m, cnt);
+        } else if (use_tv || fan < 32) {
+            pair_children<true>(a, ctl, T, S, s_tv, use_tv, sp, se, reinterpret_cast<unsigned *>(lists), 256u, meta, pi, fan,
+                                only, t, kEvalThreads, cnt);
+        } else {
+            direct_children(a, ctl, T, S, sp, se, meta, pi, fan, t, kEvalThreads, cnt);
+        }
+        add_counts(a, sys, cnt);
+    }
+    if (warp == 0) add_parents(a, sys, depth, 1u, over ? 0ull : (unsigned long long)fan);
+    __syncthreads();   // the parent's arrays and s_flag are rewritten for the next parent
+}
+
+// Children of the popped parents.  A narrow sweep (no more parents than blocks) gives each
+// block a parent at a time.  A wide one gives each warp a parent at a time from a shared
+// cursor, and then each block the parents of the systems whose table or number of children
+// asks for a block.
 __global__ void __launch_bounds__(kEvalThreads, 3) k_eval(SweepArgs a) {
     extern __shared__ __align__(16) char s_blob[];
-    float4 *s_tv_base = reinterpret_cast<float4 *>(s_blob + (a.single ? a.blob_smem : 0));
+    float4 *s_tv = reinterpret_cast<float4 *>(s_blob + (a.single ? a.blob_smem : 0));
     __shared__ double s_p[kEvalWarps][3][kMaxVars];
     __shared__ float s_f[kEvalWarps][4][kMaxVars];
     __shared__ float s_e[kEvalWarps][6][kMaxVars];
+    __shared__ __align__(8) uint16_t s_list[kEvalWarps * 256];
+    __shared__ unsigned s_need[kEvalWarps];
     __shared__ int s_flag;
     const unsigned lane = lane_id();
     const int w = threadIdx.x >> 5;
     WaveCtl *ctl = a.ctl;
     const int64_t base = ctl->base, K = ctl->k;
-    const bool block_mode = K <= (int64_t)gridDim.x;
+    const bool narrow = K <= (int64_t)gridDim.x;
+    const bool block_pass = narrow || (a.eval_forms & 2), warp_pass = !narrow && (a.eval_forms & 1);
     // blocks beyond what K parents need leave at once (the others take every parent), so
     // a small sweep does not pay for the whole grid
-    if (block_mode ? (int64_t)blockIdx.x >= K : (int64_t)blockIdx.x * (blockDim.x >> 5) >= K) return;
+    if (block_pass ? (int64_t)blockIdx.x >= K : (int64_t)blockIdx.x * kEvalWarps >= K) return;
     if (a.single) {
         const DevSys &S0 = a.tb.sys[0];
         copy_blob(s_blob, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);
         __syncthreads();
     }
-    if (block_mode) {
-        for (int64_t p = blockIdx.x; p < K; p += gridDim.x)
-            eval_parent<true>(a, ctl, s_blob, s_tv_base, s_p[0], s_f[0], s_e[0], &s_flag, parent_index(a, base, p),
-                              threadIdx.x, blockDim.x);
+    if (warp_pass) {
+        float4 *tv = s_tv + (size_t)w * (a.tv_entries / kEvalWarps);
+        WarpTally tally{-1, 0, 0u, 0ull, EvalCount{0u, 0u, 0u, 0u}};
+        for (;;) {
+            int p = 0;
+            if (lane == 0) p = atomicAdd(&ctl->cursor, 1);
+            p = __shfl_sync(kFull, p, 0);
+            if (p >= K) break;
+            eval_warp(a, ctl, s_blob, tv, s_p[w], s_f[w], s_e[w], s_list + w * 256, parent_index(a, base, p), tally);
+        }
+        flush_tally(a, tally);
+        if (!block_pass) return;
+        __syncthreads();
+    }
+    if (!warp_pass) {
+        for (int64_t p = blockIdx.x; p < K; p += gridDim.x) {
+            const int64_t pi = parent_index(a, base, p);
+            if (!(a.eval_forms & 4)) {
+                eval_block(a, ctl, s_blob, s_tv, s_p[0], s_f[0], s_e[0], s_list, &s_flag, pi);
+            } else if (w == 0) {
+                // parents of up to 8 children: a warp each, without the block's barriers
+                WarpTally tally{-1, 0, 0u, 0ull, EvalCount{0u, 0u, 0u, 0u}};
+                eval_warp(a, ctl, s_blob, s_tv, s_p[0], s_f[0], s_e[0], s_list, pi, tally);
+                flush_tally(a, tally);
+            }
+        }
         return;
     }
-    float4 *s_tv = s_tv_base + (size_t)w * a.tv_stride;
-    for (;;) {
-        int p = 0;
-        if (lane == 0) p = atomicAdd(&ctl->cursor, 1);
-        p = __shfl_sync(kFull, p, 0);
-        if (p >= K) break;
-        eval_parent<false>(a, ctl, s_blob, s_tv, s_p[w], s_f[w], s_e[w], &s_flag, parent_index(a, base, p), lane, 32u);
+    // the parents that the warps left, 256 of the block's at a time
+    for (int64_t p0 = blockIdx.x; p0 < K; p0 += (int64_t)gridDim.x * kEvalThreads) {
+        const int64_t p = p0 + (int64_t)threadIdx.x * gridDim.x;
+        const bool need = p < K && block_form(a, a.tb.sys[a.q.sys[parent_index(a, base, p)]]);
+        const unsigned bal = __ballot_sync(kFull, need);
+        if (lane == 0) s_need[w] = bal;
+        __syncthreads();
+        for (int v = 0; v < kEvalWarps; v++)
+            for (unsigned bits = s_need[v]; bits; bits &= bits - 1u)
+                eval_block(a, ctl, s_blob, s_tv, s_p[0], s_f[0], s_e[0], s_list, &s_flag,
+                           parent_index(a, base, p0 + (int64_t)(v * 32 + __ffs(bits) - 1) * gridDim.x));
+        __syncthreads();
     }
 }
 
@@ -765,7 +1146,7 @@ static cudaError_t launch_hs(const SweepArgs &a, int n, int num_sms, cudaStream_
 }
 
 size_t eval_smem_bytes(const SweepArgs &a) {
-    return (size_t)(a.single ? a.blob_smem : 0) + (size_t)a.eval_warps * a.tv_stride * sizeof(float4);
+    return (size_t)(a.single ? a.blob_smem : 0) + (size_t)a.tv_entries * sizeof(float4);
 }
 
 cudaError_t allow_max_dynamic_smem(const void *func) {
@@ -799,7 +1180,7 @@ static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int
     if (ev) cudaEventRecord(ev[0], st);
     k_wave_begin<<<1, kBeginThreads, kBeginSmem, st>>>(a);
     if (ev) cudaEventRecord(ev[1], st);
-    k_eval<<<eval_blocks, a.eval_warps * 32, eval_smem_bytes(a), st>>>(a);
+    k_eval<<<eval_blocks, kEvalThreads, eval_smem_bytes(a), st>>>(a);
     if (ev) cudaEventRecord(ev[2], st);
     k_eval64<<<num_sms * 4, kEval64Threads, head, st>>>(a);
     if (ev) cudaEventRecord(ev[3], st);

@@ -36,25 +36,39 @@ struct SweepArgs {
     int32_t single;              // 1: one system; kernels cache its blob in shared memory
     int32_t blob_smem;           // bytes of that blob
     int32_t head_smem;           // bytes of its head, all that the contraction's kernels cache
-    int32_t tv_stride;           // term-combination entries per warp region (0: no tables)
-    int32_t eval_warps;          // warps per block of k_eval
+    int32_t tv_entries;          // table entries of a block of k_eval (0: no tables)
+    int32_t eval_forms;          // bit 0: some system's parents go to warps, bit 1: to blocks;
+                                 // bit 2: every parent has few children (a warp also in narrow sweeps)
     int32_t screen;              // 1: some system may be screened in FP32 (ivs_screen.cuh)
     DevRegions rg;               // serving: per-system queue regions (rg.n == 0: shared stack)
 };
 
 // dynamic shared memory of k_eval (blob cache + the warps' combination tables) and the
-// kernels' limits; tv_stride / eval_warps come from choose_eval_layout
+// kernels' limits
 size_t eval_smem_bytes(const SweepArgs &a);
 cudaError_t configure_eval_kernels(const SweepArgs &a);
 // raises a kernel's dynamic shared memory limit to the device maximum (idempotent)
 cudaError_t allow_max_dynamic_smem(const void *func);
-// picks eval_warps and tv_stride for the largest table `max_tv` of the plan's systems
-inline void choose_eval_layout(SweepArgs &a, int max_tv) {
-    const size_t budget = 200 * 1024 - (size_t)(a.single ? a.blob_smem : 0);
-    int warps = 8;
-    while (warps > 1 && (size_t)warps * (size_t)max_tv * 16 > budget) warps--;
-    a.eval_warps = warps;
-    a.tv_stride = ((size_t)max_tv * 16 <= budget) ? max_tv : 0;
+// k_eval's table region: eight warps' tables where they fit 56 KB (three blocks per SM with
+// the blob of an n = 8 system beside them), else one table per block; a table has at most
+// 2048 entries.  sys == nullptr: any systems (the server).
+constexpr int kTvEntries = 3584;
+inline bool eval_uses_table(const DevSys &d) { return d.n_tv > 0 && (d.shadow || !d.prefilter); }
+inline void choose_eval_layout(SweepArgs &a, const DevSys *sys, int n_sys) {
+    a.tv_entries = sys ? 0 : kTvEntries;
+    a.eval_forms = sys ? 0 : 3;
+    for (int s = 0; s < n_sys; s++) {
+        const DevSys &d = sys[s];
+        if (!eval_uses_table(d)) continue;
+        const int need = (!d.eval_block && d.n_tv * 8 <= kTvEntries) ? d.n_tv * 8 : d.n_tv;
+        if (need > a.tv_entries) a.tv_entries = need;
+    }
+    bool few = sys != nullptr;
+    for (int s = 0; s < n_sys; s++) {
+        a.eval_forms |= (sys[s].eval_block || sys[s].n_tv > a.tv_entries / 8) ? 2 : 1;
+        few = few && (sys[s].bisect || sys[s].n <= 3) && sys[s].n_tv <= 64 && sys[s].m <= 8;
+    }
+    if (few && a.eval_forms == 1) a.eval_forms |= 4;
 }
 // one sweep; ev (nullable) receives n_hs_dims + 5 stage events; *kernels (nullable) the
 // number of kernels launched

@@ -339,7 +339,7 @@ extern "C" int ivs_solve_noalloc(const ivs_system *s, const double *box_lo, cons
     NA_TRY(cudaMemcpyAsync(d_depth, &rd, 4, cudaMemcpyHostToDevice, st));
     // the array keeps the previous call's contents: clear what must start at zero
     NA_TRY(cudaMemsetAsync(d_stats, 0, (size_t)ST_COUNT * 8, st));
-    choose_eval_layout(a, 0);
+    choose_eval_layout(a, &d, 1);
     NA_TRY(configure_eval_kernels(a));
     NA_TRY(launch_seed_roots(a, d_lo, d_hi, d_depth, 1, n, st));   // also resets the control block
 

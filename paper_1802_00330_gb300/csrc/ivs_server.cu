@@ -210,7 +210,7 @@ int ivs_server::init() {
     CUDA_TRY(cudaMemsetAsync(a.stats, 0, (size_t)S * ST_COUNT * sizeof(unsigned long long), stream));
     CUDA_TRY(launch_seed_roots(a, d_rlo, d_rhi, d_rdepth, 0, n_max, stream));   // empty queue, reset control
     a.screen = 1;
-    choose_eval_layout(a, 2048);   // any admitted system's table fits (hostcore caps it at 2048)
+    choose_eval_layout(a, nullptr, 0);   // any admitted system's table fits a block
     CUDA_TRY(configure_eval_kernels(a));
     for (int n = 1; n <= n_max; n++) dims.push_back(n);
     CUDA_TRY(build_sweep_graph(a, dims.data(), (int)dims.size(), num_sms * 8, 256, num_sms, &graph));

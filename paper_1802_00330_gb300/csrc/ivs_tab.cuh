@@ -41,7 +41,7 @@ __host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 
     L.head = o;
     L.tv_off = o;    o += 4u * (TF + 1);
     L.tv_map = o;    o += 4u * E;
-    L.cix = o;       o += (2u * CX + 3u) & ~3u;
+    L.cix = o;       o += ((uint32_t)CX + 3u) & ~3u;
     L.bytes = (o + 15u) & ~15u;
     return L;
 }
@@ -64,9 +64,10 @@ struct SysTab {
     const float *clo32, *chi32;
     const int32_t *poly_off; // [P + 1] term ranges
     const uint32_t *tinfo;   // term info words (above)
-    const int32_t *tv_off;   // [TF + 1]: first combination entry of each F term
+    const int32_t *tv_off;   // [TF]: first combination entry of each F term
     const uint32_t *tv_map;  // [E]: term << 8 | combination of its variables' halves
-    const uint16_t *cix;     // [TF << n] (if present): entry of F term t for child c at (t << n) + c
+    const uint8_t *cix;      // [TF << L], L = min(n, 8) (if present): the part that the low L bits
+                             // c of a child have in its combination, at (t << L) + c
     const uint8_t *fac;
 };
 
@@ -82,7 +83,7 @@ __device__ __forceinline__ SysTab make_tab(const char *blob, const DevSys &S) {
     t.tinfo = reinterpret_cast<const uint32_t *>(blob + L.tinfo);
     t.tv_off = reinterpret_cast<const int32_t *>(blob + L.tv_off);
     t.tv_map = reinterpret_cast<const uint32_t *>(blob + L.tv_map);
-    t.cix = reinterpret_cast<const uint16_t *>(blob + L.cix);
+    t.cix = reinterpret_cast<const uint8_t *>(blob + L.cix);
     t.fac = reinterpret_cast<const uint8_t *>(blob + L.fac);
     return t;
 }
@@ -224,7 +225,8 @@ __device__ __forceinline__ float4 term_shadow(const SysTab &T, int t, const Coor
         fc = T.fac[f0 + f];
         prod = sh_mul(prod, sh_pow(x(fc >> 4, f), (int)(fc & 15u), poison), poison);
     }
-    const shv v = sh_mul(shv{ce.x, ce.y, ce.z, ce.w}, prod, poison);
+    // a point coefficient that float holds exactly: one product per end, sh_mul's values
+    const shv v = ce.x == ce.w ? sh_scale(ce.x, prod, poison) : sh_mul(shv{ce.x, ce.y, ce.z, ce.w}, prod, poison);
     if (poison) {
         const float nan = __int_as_float(0x7FC00000);
         return make_float4(nan, nan, nan, nan);
@@ -232,80 +234,20 @@ __device__ __forceinline__ float4 term_shadow(const SysTab &T, int t, const Coor
     return make_float4(v.ld, v.lu, v.hd, v.hu);
 }
 
-// FP32 shadow decision of child c from its parent's table tv (same result as
-// decide_shadow on the child): 0 exclude, 1 keep, 2 undecided.  The entry of a term for
-// the child is read from the child-index table when the blob has one (small n), else
-// gathered from the child's bits in the term's variables.
-__device__ __forceinline__ int decide_from_table(const SysTab &T, const DevSys &S, const float4 *tv, unsigned c) {
-    bool undecided = false;
-    for (int i = 0; i < S.m; i++) {
-        const int t0 = T.poly_off[S.f_poly + i], t1 = T.poly_off[S.f_poly + i + 1];
-        shv acc = {0.f, 0.f, 0.f, 0.f};
-        for (int t = t0; t < t1; t++) {
-            int e;
-            if (S.n_cix > 0) {
-                e = T.cix[((unsigned)t << S.n) + c];
-            } else {
-                const uint32_t info = T.tinfo[t];
-                const int nf = term_nf(info), f0 = term_f0(info);
-                unsigned q = 0;
-                for (int f = 0; f < nf; f++) q |= ((c >> (T.fac[f0 + f] >> 4)) & 1u) << f;
-                e = T.tv_off[t] + (int)q;
-            }
-            const float4 v = tv[e];
-            const shv sv = {v.x, v.y, v.z, v.w};
-            acc = (t == t0) ? sv : sh_add(acc, sv);
-        }
-        if (acc.ld > 0.0f || acc.hu < 0.0f) return 0;
-        if (!(acc.lu <= 0.0f && acc.hd >= 0.0f)) undecided = true;   // also NaN (poison)
+// The FP64 value of term t for the same combinations, as term64 computes it.
+template <class Coord>
+__device__ __forceinline__ ivd term_combo64(const SysTab &T, int t, const Coord &x) {
+    const ivd cf = {T.clo[t], T.chi[t]};
+    const uint32_t info = T.tinfo[t];
+    const int nf = term_nf(info), f0 = term_f0(info);
+    if (nf == 0) return cf;
+    unsigned fc = T.fac[f0];
+    ivd prod = iv_pow(x(fc >> 4, 0), (int)(fc & 15u));
+    for (int f = 1; f < nf; f++) {
+        fc = T.fac[f0 + f];
+        prod = iv_mul(prod, iv_pow(x(fc >> 4, f), (int)(fc & 15u)));
     }
-    return undecided ? 2 : 1;
-}
-
-// The same decision for K children c[0..K) of one parent at once (child-index table
-// present), each exactly as decide_from_table: the K sums of an equation are independent
-// chains of loads and adds, so one thread overlaps their latencies.  An equation is
-// evaluated while any wanted child is undecided; a decided child's sums are ignored.
-// want[k] = false: c[k] is not a child (d[k] = 0).
-template <int K>
-__device__ __forceinline__ void decide_from_table_k(const SysTab &T, const DevSys &S, const float4 *tv,
-                                                    const unsigned (&c)[K], const bool (&want)[K], int (&d)[K]) {
-    int rs[K];      // -1: no equation excluded yet
-    bool und[K];
-    int open = 0;
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-        rs[k] = want[k] ? -1 : 0;
-        und[k] = false;
-        open += want[k] ? 1 : 0;
-    }
-    for (int i = 0; i < S.m && open > 0; i++) {
-        const int t0 = T.poly_off[S.f_poly + i], t1 = T.poly_off[S.f_poly + i + 1];
-        shv acc[K];
-#pragma unroll
-        for (int k = 0; k < K; k++) acc[k] = shv{0.f, 0.f, 0.f, 0.f};
-        for (int t = t0; t < t1; t++) {
-            const uint16_t *row = T.cix + ((unsigned)t << S.n);
-#pragma unroll
-            for (int k = 0; k < K; k++) {
-                const float4 v = tv[row[c[k]]];
-                const shv s = {v.x, v.y, v.z, v.w};
-                acc[k] = (t == t0) ? s : sh_add(acc[k], s);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < K; k++) {
-            if (rs[k] >= 0) continue;
-            if (acc[k].ld > 0.0f || acc[k].hu < 0.0f) {
-                rs[k] = 0;
-                open--;
-            } else if (!(acc[k].lu <= 0.0f && acc[k].hd >= 0.0f)) {
-                und[k] = true;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < K; k++) d[k] = rs[k] >= 0 ? rs[k] : (und[k] ? 2 : 1);
+    return (info & kTermPoint) ? iv_smul(cf.lo, prod) : iv_mul(cf, prod);
 }
 
 }  // namespace ivs
