@@ -1056,8 +1056,12 @@ __global__ void __launch_bounds__(kEvalThreads, 3) k_eval(SweepArgs a) {
     }
 }
 
-// FP64 evaluation of the candidates (undecided by the FP32 stage), one thread each,
-// 32 per warp from an atomic cursor so the work is dense and spread over all SMs.
+// FP64 evaluation of the candidates (undecided by the FP32 stage), 32 / g per warp from an
+// atomic cursor.  Few candidates (a sweep with the FP32 shadow leaves some hundred): g = 8
+// lanes share a candidate's equations, so the kernel takes one or two equations' chains
+// instead of all of them one after the other (n = 8: 26 -> 15 us a sweep, n = 7: 25 -> 13).  Many: one lane each (g = 1), which
+// stops at the first equation that excludes, so the FP64 pipe does no more than it has to.
+constexpr int64_t kSplitCandidates = 16384;
 __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
     extern __shared__ __align__(16) char s_blob[];
     __shared__ double sX[2 * kMaxVars * kEval64Threads];
@@ -1065,7 +1069,9 @@ __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
     double *X = sX + tid;
     WaveCtl *ctl = a.ctl;
     const int64_t count = ctl->cand_count;
-    if ((int64_t)blockIdx.x * blockDim.x >= count) return;   // not needed for this many candidates
+    const bool split = count <= kSplitCandidates;
+    // not needed for this many candidates
+    if ((int64_t)blockIdx.x * blockDim.x >= (split ? 8 * count : count)) return;
     if (a.single) {
         const DevSys &S0 = a.tb.sys[0];
         copy_blob(s_blob, a.tb.blobs + S0.blob_off, (uint32_t)S0.head_bytes);
@@ -1073,16 +1079,18 @@ __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
     }
     const unsigned lane = lane_id();
     for (;;) {
+        // candidates of the warp: 32, or 4 with 8 lanes each (equations lane, lane + 8, ...)
+        const int per = split ? 4 : 32;
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd((unsigned long long *)&ctl->cand_cursor, 32ull);
+        if (lane == 0) base = atomicAdd((unsigned long long *)&ctl->cand_cursor, (unsigned long long)per);
         base = __shfl_sync(kFull, base, 0);
         if ((long long)base >= count) break;
-        const int64_t idx = (int64_t)base + lane;
-        const bool active = idx < count;
+        const int64_t idx = (int64_t)base + (split ? lane >> 3 : lane);
+        const bool there = idx < count;
         bool keep = false;
         int sys = 0, n = 0;
         Surv sv{0, 0};
-        if (active) {
+        if (there) {
             sv = a.cand[idx];
             const int64_t pi = sv.parent;
             sys = a.q.sys[pi];
@@ -1094,7 +1102,23 @@ __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
                 X[(2 * j) * T] = up ? a.q.mid[j * a.q.cap + pi] : a.q.lo[j * a.q.cap + pi];
                 X[(2 * j + 1) * T] = up ? a.q.hi[j * a.q.cap + pi] : a.q.mid[j * a.q.cap + pi];
             }
-            keep = keep64(Tb, S, BoxCoord{X, T});
+            if (split) {
+                keep = true;
+                for (int i = (int)(lane & 7u); i < S.m; i += 8) {
+                    const ivd F = poly64(Tb, S.f_poly + i, BoxCoord{X, T});
+                    keep = keep && !(d_pos(F.lo) || d_neg(F.hi));
+                }
+            } else {
+                keep = keep64(Tb, S, BoxCoord{X, T});
+            }
+        }
+        __syncwarp();
+        bool active = there;
+        if (split) {   // a candidate's first lane speaks for it
+            const unsigned kept = __ballot_sync(kFull, keep);
+            keep = ((kept >> (lane & 24u)) & 255u) == 255u;
+            active = there && (lane & 7u) == 0u;
+            keep = keep && active;
         }
         const int sys0 = __shfl_sync(kFull, sys, 0);
         const int n0 = __shfl_sync(kFull, n, 0);
