@@ -102,57 +102,86 @@ cudaError_t scan_exclusive(const int64_t *in, int64_t *out, int64_t count, int64
 }
 
 // ---- bitonic sort of 128-bit keys ----------------------------------------------------------
-constexpr int kSortBlock = 1024;   // elements per shared-memory stage
+// 2^18 keys: 0.44 -> 0.31 ms a sort.  Every thread of a step holds a pair (element index from
+// the pair index), blocks of 2048 keys sort in shared memory, and a global pass does two
+// steps on four keys per thread, so a merge of 2^18 keys reads the keys 4 times, not 8.
+constexpr int kSortBlock = 2048;     // elements per shared-memory stage
+constexpr int kSortThreads = kSortBlock / 2;
+
+// element x of a pair / quad with its partner at distance j: bit log2(j) of the index is 0
+__device__ __forceinline__ int64_t pair_low(int64_t p, int64_t j) { return 2 * p - (p & (j - 1)); }
+__device__ __forceinline__ void order_keys(Key &x, Key &y, bool up) {
+    if (up ? key_less(y, x) : key_less(x, y)) {
+        const Key t = x;
+        x = y;
+        y = t;
+    }
+}
 
 __global__ void k_bitonic_global(Key *k, int64_t N, int64_t j, int64_t kk) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= N) return;
-    const int64_t l = i ^ j;
-    if (l <= i) return;
-    const Key x = k[i], y = k[l];
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= N / 2) return;
+    const int64_t i = pair_low(p, j);
+    Key x = k[i], y = k[i + j];
+    order_keys(x, y, (i & kk) == 0);
+    k[i] = x;
+    k[i + j] = y;
+}
+
+// steps j and j / 2 of merge size kk
+__global__ void k_bitonic_global2(Key *k, int64_t N, int64_t j, int64_t kk) {
+    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= N / 4) return;
+    const int64_t h = j / 2, i = pair_low(pair_low(p, h), j);
     const bool up = (i & kk) == 0;
-    if (up ? key_less(y, x) : key_less(x, y)) {
-        k[i] = y;
-        k[l] = x;
-    }
+    Key a = k[i], b = k[i + h], c = k[i + j], d = k[i + j + h];
+    order_keys(a, c, up);
+    order_keys(b, d, up);
+    order_keys(a, b, up);
+    order_keys(c, d, up);
+    k[i] = a;
+    k[i + h] = b;
+    k[i + j] = c;
+    k[i + j + h] = d;
 }
 
 // stages j = jmax .. 1 of merge size kk inside blocks of kSortBlock elements; with
 // kk = 0 the whole sort of every block (kk = 2 .. kSortBlock)
-__global__ void k_bitonic_shared(Key *k, int64_t N, int64_t kk, int64_t jmax) {
+__global__ void __launch_bounds__(kSortThreads) k_bitonic_shared(Key *k, int64_t kk, int64_t jmax) {
     __shared__ Key s[kSortBlock];
     const int64_t base = (int64_t)blockIdx.x * kSortBlock;
-    for (int t = threadIdx.x; t < kSortBlock; t += blockDim.x) s[t] = k[base + t];
+    const int t = threadIdx.x;
+    s[t] = k[base + t];
+    s[t + kSortThreads] = k[base + t + kSortThreads];
     __syncthreads();
     const int64_t k0 = kk ? kk : 2, k1 = kk ? kk : kSortBlock;
     for (int64_t q = k0; q <= k1; q <<= 1) {
         for (int64_t j = kk ? jmax : q / 2; j > 0; j >>= 1) {
-            for (int t = threadIdx.x; t < kSortBlock; t += blockDim.x) {
-                const int l = t ^ (int)j;
-                if (l > t) {
-                    const Key x = s[t], y = s[l];
-                    const bool up = ((base + t) & q) == 0;
-                    if (up ? key_less(y, x) : key_less(x, y)) {
-                        s[t] = y;
-                        s[l] = x;
-                    }
-                }
-            }
+            const int i = (int)pair_low(t, j), l = i + (int)j;
+            Key x = s[i], y = s[l];
+            order_keys(x, y, ((base + i) & q) == 0);
+            s[i] = x;
+            s[l] = y;
             __syncthreads();
         }
     }
-    for (int t = threadIdx.x; t < kSortBlock; t += blockDim.x) k[base + t] = s[t];
+    k[base + t] = s[t];
+    k[base + t + kSortThreads] = s[t + kSortThreads];
 }
 
 // sorts N keys (N a power of two >= kSortBlock) ascending
 cudaError_t bitonic_sort(Key *k, int64_t N, cudaStream_t st) {
     const unsigned blocks = (unsigned)(N / kSortBlock);
-    k_bitonic_shared<<<blocks, 512, 0, st>>>(k, N, 0, 0);
+    k_bitonic_shared<<<blocks, kSortThreads, 0, st>>>(k, 0, 0);
     for (int64_t kk = 2 * kSortBlock; kk <= N; kk <<= 1) {
         int64_t j = kk / 2;
-        for (; j >= kSortBlock; j >>= 1)
-            k_bitonic_global<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(k, N, j, kk);
-        k_bitonic_shared<<<blocks, 512, 0, st>>>(k, N, kk, j);
+        for (; j >= 2 * kSortBlock; j >>= 2)
+            k_bitonic_global2<<<(unsigned)((N / 4 + 255) / 256), 256, 0, st>>>(k, N, j, kk);
+        if (j >= kSortBlock) {
+            k_bitonic_global<<<(unsigned)((N / 2 + 255) / 256), 256, 0, st>>>(k, N, j, kk);
+            j >>= 1;
+        }
+        k_bitonic_shared<<<blocks, kSortThreads, 0, st>>>(k, kk, j);
     }
     return cudaGetLastError();
 }
@@ -163,18 +192,38 @@ __global__ void k_fill_keys(Key *k, int64_t from, int64_t to) {
 }
 
 // ---- union-find -----------------------------------------------------------------------------
+// Path halving by plain stores: an item that is not a root never becomes one again, its
+// parent only ever moves to an ancestor, and every ancestor is a valid parent, so racing
+// stores are harmless (the intermediate pointer jumping of ECL-CC, Jaiganesh and Burtscher
+// 2018).  As compare-and-swaps they queued up on the parents of a cluster's few top items.
+__device__ __forceinline__ int64_t uf_load(const int64_t *par, int64_t x) {
+    return (int64_t)*reinterpret_cast<const volatile long long *>(par + x);
+}
 __device__ __forceinline__ int64_t uf_find(int64_t *par, int64_t x) {
+    int64_t p = uf_load(par, x);
     for (int it = 0; it < kUfIters; it++) {
-        const int64_t p = par[x];
         if (p == x) return x;
-        const int64_t gp = par[p];
-        if (gp != p) atomicCAS((unsigned long long *)&par[x], (unsigned long long)p, (unsigned long long)gp);
+        const int64_t gp = uf_load(par, p);
+        if (gp == p) return p;
+        *reinterpret_cast<volatile long long *>(par + x) = (long long)gp;
+        x = gp;
+        p = uf_load(par, x);
+    }
+    return -1;
+}
+
+// the root of x without halving: k_uf_flatten's own stores must stay the last ones
+__device__ __forceinline__ int64_t uf_root(const int64_t *par, int64_t x) {
+    for (int it = 0; it < kUfIters; it++) {
+        const int64_t p = uf_load(par, x);
+        if (p == x) return x;
         x = p;
     }
     return -1;
 }
 
-// unites the sets of a and b; the root with the larger index is hooked under the smaller
+// unites the sets of a and b; the root with the larger index is hooked under the smaller.
+// (false: it gave up)
 __device__ __forceinline__ bool uf_union(int64_t *par, int64_t a, int64_t b) {
     for (int it = 0; it < kUfIters; it++) {
         a = uf_find(par, a);
@@ -198,10 +247,84 @@ __global__ void k_iota(int64_t *par, int64_t count) {
         par[i] = i;
 }
 
+// Unites touching items.  Items lie in sorted order, coordinate j of item p as integer keys
+// [lo, hi] at key[(2 j) * count + p], key[(2 j + 1) * count + p] (order-preserving images of
+// a box's ends; a cell's index c and c + 1); item p may only touch the items p + 1 .. end[p] - 1.
+// A block takes 32 items, one per lane of every warp, and its warps share the range that
+// follows them: an item of the range is read by a warp once (a broadcast) and tested against
+// 32, coordinate 1 first.  Integer compares: FP64 ones would run at 1/64 of their rate.
+// id: what the union-find calls item p (nullptr: p).  (A warp per item, its lanes gathering
+// the candidates' rows through the sorted keys, took 6.3 ms for 2e5 boxes of 6 coordinates,
+// and 1.1 ms for their 8.9e4 cells; this 1.4 and 0.47.)
+// Touching pairs queue up in shared memory and are united 32 at a time: a union is a chain
+// of dependent loads, which the lanes that found a pair would go through on their own.
+constexpr int kUniteWarps = 8;
+__device__ __forceinline__ void unite_pair(int64_t *par, const Key *id, longlong2 w, int *err) {
+    if (!uf_union(par, id ? (int64_t)id[w.x].b : w.x, id ? (int64_t)id[w.y].b : w.y)) atomicExch(err, 1);
+}
+template <class K, int N>
+__global__ void __launch_bounds__(kUniteWarps * 32) k_unite(const K *key, int64_t count, const int64_t *end, const Key *id,
+                                                            int64_t *par, int *err) {
+    __shared__ longlong2 s_pair[kUniteWarps][64];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t p0 = (int64_t)blockIdx.x * 32; p0 < count; p0 += (int64_t)gridDim.x * 32) {
+        const int64_t p = p0 + lane;
+        const bool on = p < count;
+        K l[N], h[N];
+#pragma unroll
+        for (int j = 0; j < N; j++) {
+            l[j] = on ? key[(int64_t)(2 * j) * count + p] : K(0);
+            h[j] = on ? key[(int64_t)(2 * j + 1) * count + p] : K(0);
+        }
+        const int64_t stop = on ? end[p] : 0;
+        int64_t last = stop;
+        for (int o = 16; o > 0; o >>= 1) {
+            const int64_t x = __shfl_xor_sync(0xFFFFFFFFu, last, o);
+            last = x > last ? x : last;
+        }
+        constexpr int J = N > 1 ? 1 : 0;   // the coordinate tested first
+        const K *kl = key + (int64_t)(2 * J) * count, *kh = key + (int64_t)(2 * J + 1) * count;
+        int held = 0;   // pairs in the warp's queue
+        for (int64_t q = p0 + 1 + warp; q < last; q += kUniteWarps) {
+            bool touch = kl[q] <= h[J] && l[J] <= kh[q] && q > p && q < stop;
+            if (!__any_sync(0xFFFFFFFFu, touch)) continue;
+#pragma unroll
+            for (int j = 0; j < N; j++)
+                touch = touch && key[(int64_t)(2 * j) * count + q] <= h[j] && l[j] <= key[(int64_t)(2 * j + 1) * count + q];
+            const unsigned bal = __ballot_sync(0xFFFFFFFFu, touch);
+            if (!bal) continue;
+            if (touch) s_pair[warp][held + __popc(bal & ((1u << lane) - 1u))] = make_longlong2(p, q);
+            held += __popc(bal);
+            __syncwarp();
+            if (held >= 32) {
+                const longlong2 w = s_pair[warp][held - 32 + lane];
+                held -= 32;
+                unite_pair(par, id, w, err);
+                __syncwarp();
+            }
+        }
+        if (lane < held) unite_pair(par, id, s_pair[warp][lane], err);
+        __syncwarp();
+    }
+}
+template <class K>
+cudaError_t launch_unite(int n, const K *key, int64_t count, const int64_t *end, const Key *id, int64_t *par, int *err,
+                         cudaStream_t st) {
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((count + 31) / 32, 1 << 20));
+    switch (n) {
+#define IVS_UNITE(N) case N: k_unite<K, N><<<grid, kUniteWarps * 32, 0, st>>>(key, count, end, id, par, err); break;
+        IVS_UNITE(1) IVS_UNITE(2) IVS_UNITE(3) IVS_UNITE(4) IVS_UNITE(5) IVS_UNITE(6) IVS_UNITE(7) IVS_UNITE(8)
+        IVS_UNITE(9) IVS_UNITE(10) IVS_UNITE(11) IVS_UNITE(12) IVS_UNITE(13) IVS_UNITE(14) IVS_UNITE(15) IVS_UNITE(16)
+#undef IVS_UNITE
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 // full compression; roots[i] = 1 when i is a root
 __global__ void k_uf_flatten(int64_t *par, int64_t count, int64_t *is_root, int *err) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = uf_find(par, i);
+        const int64_t r = uf_root(par, i);
         if (r < 0) {
             atomicExch(err, 1);
             continue;
@@ -233,12 +356,15 @@ __device__ __forceinline__ void cell_range(const BoxView &v, const Grid &g, int6
     b = (int32_t)y;
 }
 
-__global__ void k_bt_count(BoxView v, Grid g, int64_t max_cells, int64_t *m, int *over) {
+// the cells per box; the ranges stay for k_bt_emit (coordinate j of box i at j * count + i):
+// their divisions are the FP64 part of both
+__global__ void k_bt_count(BoxView v, Grid g, int64_t max_cells, int64_t *m, int2 *range, int *over) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < v.count; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t c = 1;
         for (int j = 0; j < v.n; j++) {
             int32_t a, b;
             cell_range(v, g, i, j, a, b);
+            range[(int64_t)j * v.count + i] = make_int2(a, b);
             c *= (int64_t)(b - a + 1);
             if (c > max_cells) {
                 atomicExch(over, 1);
@@ -270,12 +396,14 @@ __device__ __forceinline__ int32_t key_get(Key k, const Grid &g, int n, int j) {
     return (int32_t)(v & mask);
 }
 
-__global__ void k_bt_emit(BoxView v, Grid g, const int64_t *offs, Key *keys) {
+__global__ void k_bt_emit(BoxView v, Grid g, const int64_t *offs, const int2 *range, Key *keys) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < v.count; i += (int64_t)gridDim.x * blockDim.x) {
         int32_t a[kMaxVars], b[kMaxVars], cur[kMaxVars];
         int64_t m = 1;
         for (int j = 0; j < v.n; j++) {
-            cell_range(v, g, i, j, a[j], b[j]);
+            const int2 r = range[(int64_t)j * v.count + i];
+            a[j] = r.x;
+            b[j] = r.y;
             cur[j] = a[j];
             m *= (int64_t)(b[j] - a[j] + 1);
         }
@@ -334,21 +462,15 @@ __global__ void k_bt_ranges(const Key *u, int64_t d, Grid g, int n, int64_t *end
     }
 }
 
-// one warp per cell: unite it with the candidates whose indices differ by <= 1 everywhere
-__global__ void k_bt_unite(const Key *u, int64_t d, Grid g, int n, const int64_t *end, int64_t *par, int *err) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t p = warp; p < d; p += warps) {
-        int32_t c[kMaxVars];
-        for (int j = 0; j < n; j++) c[j] = key_get(u[p], g, n, j);
-        for (int64_t q = p + 1 + lane; q < end[p]; q += 32) {
-            bool touch = true;
-            for (int j = 0; j < n && touch; j++) {
-                const int32_t x = key_get(u[q], g, n, j);
-                touch = x - c[j] <= 1 && c[j] - x <= 1;
-            }
-            if (touch && !uf_union(par, p, q)) atomicExch(err, 1);
+// the cells' indices as k_unite's keys: cells touch when their indices differ by <= 1
+// everywhere, i.e. when the closed intervals [c, c + 1] meet
+__global__ void k_bt_planes(const Key *u, int64_t d, Grid g, int n, int32_t *key) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < d; p += (int64_t)gridDim.x * blockDim.x) {
+        const Key k = u[p];
+        for (int j = 0; j < n; j++) {
+            const int32_t c = key_get(k, g, n, j);
+            key[(int64_t)(2 * j) * d + p] = c;
+            key[(int64_t)(2 * j + 1) * d + p] = c + 1;
         }
     }
 }
@@ -394,17 +516,14 @@ __global__ void k_cl_ranges(BoxView v, const Key *k, int64_t *end, int64_t *work
     }
 }
 
-__global__ void k_cl_unite(BoxView v, const Key *k, const int64_t *end, int64_t *par, int *err) {
-    const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t p = warp; p < v.count; p += warps) {
+// the boxes' ends in sorted order as k_unite's keys; a NaN end compares with nothing
+__global__ void k_cl_planes(BoxView v, const Key *k, unsigned long long *key) {
+    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < v.count; p += (int64_t)gridDim.x * blockDim.x) {
         const int64_t i = (int64_t)k[p].b;
-        for (int64_t q = p + 1 + lane; q < end[p]; q += 32) {
-            const int64_t o = (int64_t)k[q].b;
-            bool touch = true;
-            for (int j = 0; j < v.n && touch; j++) touch = v.l(o, j) <= v.h(i, j) && v.l(i, j) <= v.h(o, j);
-            if (touch && !uf_union(par, i, o)) atomicExch(err, 1);
+        for (int j = 0; j < v.n; j++) {
+            const double l = v.l(i, j), h = v.h(i, j);
+            key[(int64_t)(2 * j) * v.count + p] = isnan(l) ? ~0ull : dkey(l);
+            key[(int64_t)(2 * j + 1) * v.count + p] = isnan(h) ? 0ull : dkey(h);
         }
     }
 }
@@ -498,8 +617,10 @@ int backtrack_device(const BoxView &v, const double *box_lo, const double *box_h
     RT_TRY(sc.get(&offs, v.count));
     RT_TRY(sc.get(&tot, 2));
     RT_TRY(sc.get(&flags, 2));
+    int2 *range = nullptr;
+    RT_TRY(sc.get(&range, (size_t)v.count * n));
     RT_TRY(cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
-    k_bt_count<<<grid_for(v.count), 256, 0, st>>>(v, g, max_cells, m, flags);
+    k_bt_count<<<grid_for(v.count), 256, 0, st>>>(v, g, max_cells, m, range, flags);
     RT_TRY(cudaGetLastError());
     RT_TRY(scan_exclusive(m, offs, v.count, tot, st, sc.v));
     int64_t total = 0;
@@ -512,7 +633,7 @@ int backtrack_device(const BoxView &v, const double *box_lo, const double *box_h
     Key *keys = nullptr, *uniq = nullptr;
     int64_t *fl = nullptr, *pos = nullptr;
     RT_TRY(sc.get(&keys, N));
-    k_bt_emit<<<grid_for(v.count), 128, 0, st>>>(v, g, offs, keys);
+    k_bt_emit<<<grid_for(v.count), 128, 0, st>>>(v, g, offs, range, keys);
     k_fill_keys<<<grid_for(N - total), 256, 0, st>>>(keys, total, N);
     RT_TRY(cudaGetLastError());
     RT_TRY(bitonic_sort(keys, N, st));
@@ -541,8 +662,11 @@ int backtrack_device(const BoxView &v, const double *box_lo, const double *box_h
     RT_TRY(cudaMemcpyAsync(&hw, wsum, sizeof(hw), cudaMemcpyDeviceToHost, st));
     RT_TRY(cudaStreamSynchronize(st));
     if ((double)hw > kMaxPairTests) return fail(IVS_ERR_BUDGET, "ivs_backtrack: too many cells to group");
+    int32_t *key = nullptr;
+    RT_TRY(sc.get(&key, (size_t)d * 2 * n));
     k_iota<<<grid_for(d), 256, 0, st>>>(par, d);
-    k_bt_unite<<<grid_for(d * 32), 256, 0, st>>>(uniq, d, g, n, end, par, flags + 1);
+    k_bt_planes<<<grid_for(d), 256, 0, st>>>(uniq, d, g, n, key);
+    RT_TRY(launch_unite<int32_t>(n, key, d, end, nullptr, par, flags + 1, st));
     int64_t *root = work;   // reused
     k_uf_flatten<<<grid_for(d), 256, 0, st>>>(par, d, root, flags + 1);
     RT_TRY(cudaGetLastError());
@@ -584,8 +708,11 @@ int clusters_device(const BoxView &v, int64_t *n_clusters, int64_t *label_h, dou
     RT_TRY(cudaMemcpyAsync(&hw, wsum, sizeof(hw), cudaMemcpyDeviceToHost, st));
     RT_TRY(cudaStreamSynchronize(st));
     if ((double)hw > kMaxPairTests) return fail(IVS_ERR_BUDGET, "ivs_clusters: too many overlapping boxes");
+    unsigned long long *key = nullptr;
+    RT_TRY(sc.get(&key, (size_t)v.count * 2 * v.n));
     k_iota<<<grid_for(v.count), 256, 0, st>>>(par, v.count);
-    k_cl_unite<<<grid_for(v.count * 32), 256, 0, st>>>(v, keys, end, par, err);
+    k_cl_planes<<<grid_for(v.count), 256, 0, st>>>(v, keys, key);
+    RT_TRY(launch_unite<unsigned long long>(v.n, key, v.count, end, keys, par, err, st));
     k_uf_flatten<<<grid_for(v.count), 256, 0, st>>>(par, v.count, nullptr, err);
     // clusters numbered in the order of their first box
     RT_TRY(sc.get(&num, v.count));
