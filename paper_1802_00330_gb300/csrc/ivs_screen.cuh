@@ -377,6 +377,9 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
         {
             const int b = t / WD, j = t % WD;
             const int jc = j < N ? j : N - 1;   // idle lanes shadow the last column
+            // boxes that still want the sweep: in range, not settled by the centred form
+            const bool want = (s_mode[b] & 2) && !s_bad[b] && !(s_fate[b] & 3);
+            const bool any = __any_sync(kFull, want);
             float gm[N], gr[N];
 #pragma unroll
             for (int i = 0; i < N; i++) {
@@ -385,6 +388,7 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
                 if (sf[C::JR + (i * N + jc) * P + b] <= kTiny) gr[i] = kTiny;   // an exact constant
             }
             __syncthreads();   // J's half widths and radii have been read: B's columns take their place
+            if (any) {   // (a warp whose boxes are all settled skips the rest)
             float *col1 = sf + C::G1 + b * C::GS, *col2 = sf + C::G2 + b * C::GS;
             unsigned used = 0;
             bool ok = true;
@@ -525,6 +529,7 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
                 }
                 if (v == 1) atomicOr(&s_fate[b], 4);
                 else if (v == 0) atomicOr(&s_fate[b], 8);
+            }
             }
         }
         __syncthreads();
