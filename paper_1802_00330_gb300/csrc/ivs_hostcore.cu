@@ -85,6 +85,23 @@ void add_term(SysBuild &b, double clo, double chi, const uint8_t *e, int n) {
 // combination of its variables' halves (2^factors entries), when the total stays small.
 constexpr int kMaxTermCombos = 2048;
 
+ScrTerm screen_term(double clo, double chi, uint32_t info, const uint8_t *fac, int terms) {
+    ScrTerm q{to_float_down(clo), 0.0f, 0xFFFFFFFFu, 0u};
+    const int nf = term_nf(info), f0 = term_f0(info);
+    int deg = 0;
+    bool simple = nf <= 3 && clo == chi;
+    for (int f = 0; f < nf; f++) {
+        const int k = fac[f0 + f] & 15;
+        deg += k;
+        simple = simple && k <= kScrPow;
+        if (simple) q.fac = (q.fac & ~(255u << (8 * f))) | ((uint32_t)((fac[f0 + f] >> 4) * kScrPow + k - 1) << (8 * f));
+    }
+    // (rounded up: the factor covers the float products and the coefficient's own rounding)
+    q.w = to_float_up(std::max(std::fabs(clo), std::fabs(chi)) * (2.0 * deg + terms + 6.0) * (1.0 + 1e-6));
+    q.kind = !simple ? 0u : (nf == 0 && terms == 1 && (double)q.c == clo) ? 3u : 1u;
+    return q;
+}
+
 void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
     const int T = (int)b.clo.size(), P = (int)b.poly_off.size() - 1, F = (int)b.fac.size();
     // entries by the terms' number of factors and exponents, so that a warp that fills a
@@ -94,12 +111,13 @@ void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
     std::vector<uint32_t> tv_map;
     std::vector<int> by_form((size_t)n_fterms);
     for (int t = 0; t < n_fterms; t++) by_form[(size_t)t] = t;
-    auto form = [&](int t) {
-        std::vector<uint8_t> f{(uint8_t)term_nf(b.tinfo[t])};
-        for (int q = 0; q < term_nf(b.tinfo[t]); q++) f.push_back(b.fac[term_f0(b.tinfo[t]) + q] & 15u);
-        return f;
-    };
-    std::stable_sort(by_form.begin(), by_form.end(), [&](int x, int y) { return form(x) < form(y); });
+    std::vector<uint64_t> form((size_t)n_fterms);   // factors, then the exponents, 4 bits each
+    for (int t = 0; t < n_fterms; t++) {
+        form[(size_t)t] = (uint64_t)term_nf(b.tinfo[t]) << 40;
+        for (int q = 0; q < term_nf(b.tinfo[t]) && q < 8; q++)
+            form[(size_t)t] |= (uint64_t)(b.fac[term_f0(b.tinfo[t]) + q] & 15u) << (4 * q);
+    }
+    std::stable_sort(by_form.begin(), by_form.end(), [&](int x, int y) { return form[(size_t)x] < form[(size_t)y]; });
     bool tv_ok = true;
     for (int t : by_form) {
         const int nf = term_nf(b.tinfo[t]), combos = d.bisect ? 2 : 1 << nf;
@@ -136,6 +154,11 @@ void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
         std::memcpy(base + L.clo32 + 4u * t, &c32[0], 4);
         std::memcpy(base + L.chi32 + 4u * t, &c32[1], 4);
     }
+    for (int p = 0; p < P; p++)
+        for (int t = b.poly_off[p]; t < b.poly_off[p + 1]; t++) {
+            const ScrTerm q = screen_term(b.clo[t], b.chi[t], b.tinfo[t], b.fac.data(), b.poly_off[p + 1] - b.poly_off[p]);
+            std::memcpy(base + L.scr + 16u * t, &q, 16);
+        }
     if (T) {
         std::memcpy(base + L.clo, b.clo.data(), 8u * T);
         std::memcpy(base + L.chi, b.chi.data(), 8u * T);

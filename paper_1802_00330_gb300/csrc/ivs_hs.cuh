@@ -358,10 +358,16 @@ __device__ __forceinline__ void m_block(double *sd, const int *si, int t) {
 #pragma unroll
             for (int u = 0; u < N; u++) col[u] = ivd{sd[C::FR + (2 * u) * BB + b], sd[C::FR + (2 * u + 1) * BB + b]};
         }
+        // entries that are 0 for every box add nothing (a sum's zero may change its sign, which
+        // nothing reads): skipped
+        unsigned nz = 0;
+#pragma unroll
+        for (int u = 0; u < N; u++) nz |= (d_iszero(col[u].lo) && d_iszero(col[u].hi)) ? 0u : 1u << u;
         for (int i = 0; i < N; i++) {
             ivd acc = iv_smul(G[(i * N) * BB + b], col[0]);
 #pragma unroll
-            for (int u = 1; u < N; u++) acc = iv_add(acc, iv_smul(G[(i * N + u) * BB + b], col[u]));
+            for (int u = 1; u < N; u++)
+                if ((nz >> u) & 1u) acc = iv_add(acc, iv_smul(G[(i * N + u) * BB + b], col[u]));
             double *dst = (j < N) ? J + (2 * (i * N + j)) * BB + b : sd + C::FR + (2 * i) * BB + b;
             dst[0] = acc.lo;
             dst[BB] = acc.hi;

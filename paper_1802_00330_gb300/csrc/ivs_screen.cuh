@@ -78,7 +78,10 @@ struct Cfg {
     static constexpr int JEND = JR + N * N * P, GEND = G2 + BB * GS;
     static constexpr int XL = JEND > GEND ? JEND : GEND;       // N: box ends
     static constexpr int XH = XL + N * BB;
-    static constexpr int HW = XH + N * BB;                     // N: half widths
+    static constexpr int PL = XH + N * BB;                     // kScrPow N: powers' lower ends
+    static constexpr int PH = PL + kScrPow * N * BB;           // and upper ends
+    static constexpr int PX = PH + kScrPow * N * BB;           // powers of the centre
+    static constexpr int HW = PX + kScrPow * N * BB;           // N: half widths
     static constexpr int FV = HW + N * BB;                     // N: f(x)
     static constexpr int FR = FV + N * BB;                     // N: its radius
     static constexpr int VEC = (FR + N * BB + 3) & ~3;         // per box N x {W h, radius, magnitude, f}
@@ -129,12 +132,42 @@ __device__ __forceinline__ void pow32(float l, float h, float m, int k, float &a
 // Natural extension of polynomial p over the box (ends xl, xh, stride 32 floats).  The FP64
 // ends are real interval arithmetic up to rounding, so the float ends differ from them by at
 // most (operations + input roundings) x 2^-24 x the sum of the terms' magnitudes.
-__device__ __forceinline__ Poly poly_c(const SysTab &T, int p, const float *xl, const float *xh) {
+// Terms of up to three factors of degree up to kScrPow read the box's powers (pl, ph: computed
+// once per box, stride 32) and one 16-byte record; the others go through the term table.
+// (With the table alone every term decoded its factors and raised its powers again; with that, the
+// n = 11 stage 30.3 -> 23.6 ms and kinema 93.6 -> 87.4, the pivot search by trees included.)
+__device__ __forceinline__ Poly poly_c(const SysTab &T, int p, const float *xl, const float *xh, const float *pl_,
+                                       const float *ph_) {
     const int t0 = T.poly_off[p], t1 = T.poly_off[p + 1];
     const float nt = (float)(t1 - t0 + 6);
     float lo = 0.0f, hi = 0.0f, rad = 0.0f;
     bool exact = t1 - t0 <= 1;
     for (int t = t0; t < t1; t++) {
+        const ScrTerm q = T.scr[t];
+        if (q.kind) {
+            float l = 1.0f, h = 1.0f, m = 1.0f;
+            uint32_t f = q.fac;
+            if ((f & 255u) != 255u) {
+                const int at = (int)(f & 255u) * 32;
+                l = pl_[at];
+                h = ph_[at];
+                m = fmaxf(fabsf(l), fabsf(h));
+                for (f = (f >> 8) | 0xFF000000u; (f & 255u) != 255u; f = (f >> 8) | 0xFF000000u) {
+                    const int at2 = (int)(f & 255u) * 32;
+                    const float a = pl_[at2], b = ph_[at2];
+                    const float p1 = l * a, p2 = l * b, p3 = h * a, p4 = h * b;
+                    l = fminf(fminf(p1, p2), fminf(p3, p4));
+                    h = fmaxf(fmaxf(p1, p2), fmaxf(p3, p4));
+                    m *= fmaxf(fabsf(a), fabsf(b));
+                }
+            }
+            const float q1 = q.c * l, q2 = q.c * h;
+            lo += fminf(q1, q2);
+            hi += fmaxf(q1, q2);
+            rad = fmaf(q.w, m, rad);
+            exact = exact && q.kind == 3u;
+            continue;
+        }
         const uint32_t info = T.tinfo[t];
         const float4 ce = T.cs[t];
         const int nf = term_nf(info), f0 = term_f0(info);
@@ -176,11 +209,24 @@ __device__ __forceinline__ Poly poly_c(const SysTab &T, int p, const float *xl, 
 
 // value of polynomial p at the box's centre (each coordinate within 2 units of the largest
 // end's magnitude), with its radius
-__device__ __forceinline__ float2 poly_v(const SysTab &T, int p, const float *xl, const float *xh) {
+__device__ __forceinline__ float2 poly_v(const SysTab &T, int p, const float *xl, const float *xh, const float *pl_,
+                                         const float *ph_, const float *px_) {
     const int t0 = T.poly_off[p], t1 = T.poly_off[p + 1];
     const float nt = (float)(t1 - t0 + 6);
     float v = 0.0f, w = 0.0f, rad = 0.0f;
     for (int t = t0; t < t1; t++) {
+        const ScrTerm q = T.scr[t];
+        if (q.kind) {
+            float x = q.c, m = q.w;
+            for (uint32_t f = q.fac; (f & 255u) != 255u; f = (f >> 8) | 0xFF000000u) {
+                const int at = (int)(f & 255u) * 32;
+                x *= px_[at];
+                m *= fmaxf(fabsf(pl_[at]), fabsf(ph_[at]));
+            }
+            v += x;
+            rad = fmaf(2.0f, m, rad);   // the centre's powers err by at most twice the ends'
+            continue;
+        }
         const uint32_t info = T.tinfo[t];
         const float4 ce = T.cs[t];
         const int nf = term_nf(info), f0 = term_f0(info);
@@ -218,6 +264,19 @@ __device__ __forceinline__ void load_col(const float *p, float (&v)[NP]) {
         v[4 * q + 2] = x.z;
         v[4 * q + 3] = x.w;
     }
+}
+
+template <int M>
+__device__ __forceinline__ float tree_max(const float (&v)[M]) {
+    float m[M];
+#pragma unroll
+    for (int i = 0; i < M; i++) m[i] = v[i];
+#pragma unroll
+    for (int o = 1; o < M; o <<= 1) {
+#pragma unroll
+        for (int i = 0; i + o < M; i += 2 * o) m[i] = fmaxf(m[i], m[i + o]);
+    }
+    return m[0];
 }
 
 // one atomic per distinct (system, slot) of the warp's counting lanes
@@ -318,6 +377,17 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
             sf[C::XL + j * BB + b] = l;
             sf[C::XH + j * BB + b] = h;
             sf[C::HW + j * BB + b] = hw;
+#pragma unroll
+            for (int k = 1; k <= kScrPow; k++) {
+                float x, y, mm;
+                pow32(l, h, fmaxf(fabsf(l), fabsf(h)), k, x, y, mm);
+                sf[C::PL + (j * kScrPow + k - 1) * BB + b] = x;
+                sf[C::PH + (j * kScrPow + k - 1) * BB + b] = y;
+                const float c = 0.5f * (l + h);
+                float v = c;
+                for (int i = 1; i < k; i++) v *= c;
+                sf[C::PX + (j * kScrPow + k - 1) * BB + b] = v;
+            }
             sw[j * BB + b] = w;
         }
         __syncthreads();
@@ -331,12 +401,13 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
             for (int q = warp; q < N * N + N; q += NT / 32) {
                 if (!on) continue;
                 if (q < N * N) {
-                    const Poly v = poly_c(T, S.j_poly + q, xl, xh);
+                    const Poly v = poly_c(T, S.j_poly + q, xl, xh, sf + C::PL + b, sf + C::PH + b);
                     sf[C::JC + q * P + b] = v.c;
                     sf[C::JW + q * P + b] = v.w;
                     sf[C::JR + q * P + b] = v.r;
                 } else {
-                    const float2 v = poly_v(T, S.f_poly + (q - N * N), xl, xh);
+                    const float2 v = poly_v(T, S.f_poly + (q - N * N), xl, xh, sf + C::PL + b, sf + C::PH + b,
+                                            sf + C::PX + b);
                     sf[C::FV + (q - N * N) * BB + b] = v.x;
                     sf[C::FR + (q - N * N) * BB + b] = v.y;
                 }
@@ -407,35 +478,37 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
                 float f[C::NP], fr[C::NP];
                 load_col<C::NP>(col1 + k * C::NP, f);
                 load_col<C::NP>(col2 + k * C::NP, fr);
-                // the pivot: the largest of the unused rows, by more than the radii
-                int p = 0;
-                float best = -1.0f, br = 0.0f, pv = 1.0f;
+                // the pivot: the largest of the unused rows, by more than the radii.  Maxima by
+                // trees and the pivot's entries through shared memory: as chains of selects
+                // this was the longest part of a step.  (fmaxf passes a NaN over, but a NaN
+                // entry stays in its row and fails the range test at the end.)
+                float top[C::NP];
 #pragma unroll
-                for (int i = 0; i < N; i++) {
-                    const float v = fabsf(f[i]);
-                    const bool take = !((used >> i) & 1u) && v > best;
-                    best = take ? v : best;
-                    br = take ? fr[i] : br;
-                    pv = take ? f[i] : pv;
-                    p = take ? i : p;
-                }
+                for (int i = 0; i < C::NP; i++) top[i] = i < N && !((used >> i) & 1u) ? fabsf(f[i]) : -1.0f;
+                const float best = tree_max<C::NP>(top);
+                unsigned at = 0;
+#pragma unroll
+                for (int i = 0; i < N; i++) at |= top[i] == best ? 1u << i : 0u;
+                const int p = at ? __ffs((int)at) - 1 : 0;
+                const float pv = col1[k * C::NP + p], br = col2[k * C::NP + p];
                 const float low = __fsub_rd(best, br);
-                ok = ok && low > 1e-15f && best < kHuge;
 #pragma unroll
-                for (int i = 0; i < N; i++)
-                    if (!((used >> i) & 1u) && i != p) ok = ok && __fadd_ru(fabsf(f[i]), fr[i]) < low;
+                for (int i = 0; i < C::NP; i++)
+                    top[i] = i < N && i != p && !((used >> i) & 1u) ? __fadd_ru(fabsf(f[i]), fr[i]) : -1.0f;
+                ok = ok && low > 1e-15f && best < kHuge && tree_max<C::NP>(top) < low;
                 used |= 1u << p;
                 prow[k] = p;
                 // 1 / pivot, then the pivot row's entry of this column
                 const float rp = __frcp_rn(pv);
                 const float rr = fma_ru(mul_ru(br, fabsf(rp) * (1.0f + 4.0f * kU)), __frcp_ru(low),
                                         fma_ru(2.0f * kU, fabsf(rp), kTiny));
-                float am = 0.0f, ar = 0.0f;
+                unsigned ua = 0, ur = 0;   // entry p of the lane's column
 #pragma unroll
                 for (int i = 0; i < N; i++) {
-                    am = i == p ? gm[i] : am;
-                    ar = i == p ? gr[i] : ar;
+                    ua |= i == p ? __float_as_uint(gm[i]) : 0u;
+                    ur |= i == p ? __float_as_uint(gr[i]) : 0u;
                 }
+                const float am = __uint_as_float(ua), ar = __uint_as_float(ur);
                 float c = am * rp;
                 float cr = fma_ru(fabsf(am), rr, fma_ru(ar, __fadd_ru(fabsf(rp), rr), fma_ru(2.0f * kU, fabsf(c), kTiny)));
                 if (j == k) {

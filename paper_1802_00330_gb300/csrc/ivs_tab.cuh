@@ -21,7 +21,7 @@ namespace ivs {
 // byte layout of a system blob with T terms, P polynomials, F factors, TF terms in the
 // equations F_i, E term-combination entries and CX child-index entries
 struct BlobLayout {
-    uint32_t cs, clo, chi, clo32, chi32, poly_off, tinfo, fac, head, tv_off, tv_map, cix, bytes;
+    uint32_t cs, scr, clo, chi, clo32, chi32, poly_off, tinfo, fac, head, tv_off, tv_map, cix, bytes;
 };
 // The head (all that evaluates polynomials) comes first: kernels that do not read the
 // per-parent tables cache the head alone (at n = 8 5 KB of 45, a third block per SM for k_hs<8>
@@ -30,6 +30,7 @@ __host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 
     BlobLayout L;
     uint32_t o = 0;
     L.cs = o;        o += 16u * T;
+    L.scr = o;       o += 16u * T;
     L.clo = o;       o += 8u * T;
     L.chi = o;       o += 8u * T;
     L.clo32 = o;     o += 4u * T;
@@ -58,7 +59,19 @@ __host__ __device__ inline uint32_t term_info(uint32_t start, uint32_t cnt, doub
     return (start << 5) | cnt | (clo == chi ? kTermPoint : 0u);
 }
 
+// A term as the FP32 screen reads it, one 16-byte load: the coefficient, the weight of its
+// magnitude in the error radius (|c| (2 degree + terms of its polynomial + 6)), up to three
+// factors as bytes (variable * kScrPow + exponent - 1, 255: none), and a flag word: 0 general
+// (more factors, higher exponents or a coefficient interval: the term table is read), 1
+// simple, 3 simple, constant and exact in float.
+constexpr int kScrPow = 3;
+struct ScrTerm {
+    float c, w;
+    uint32_t fac, kind;
+};
+
 struct SysTab {
+    const ScrTerm *scr;
     const float4 *cs;        // {rd32(c_lo), ru32(c_lo), rd32(c_hi), ru32(c_hi)}
     const double *clo, *chi; // coefficient interval
     const float *clo32, *chi32;
@@ -75,6 +88,7 @@ __device__ __forceinline__ SysTab make_tab(const char *blob, const DevSys &S) {
     const BlobLayout L = blob_layout(S.n_terms, S.n_polys, S.n_facs, S.n_fterms, S.n_tv, S.n_cix);
     SysTab t;
     t.cs = reinterpret_cast<const float4 *>(blob + L.cs);
+    t.scr = reinterpret_cast<const ScrTerm *>(blob + L.scr);
     t.clo = reinterpret_cast<const double *>(blob + L.clo);
     t.chi = reinterpret_cast<const double *>(blob + L.chi);
     t.clo32 = reinterpret_cast<const float *>(blob + L.clo32);
