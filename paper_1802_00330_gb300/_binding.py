@@ -160,8 +160,8 @@ def _check(rc):
         raise IvsError(rc, f"{lib.ivs_status_str(rc).decode()}: {lib.ivs_last_error().decode()}")
 
 
-def _ptr(a):
-    return a.ctypes.data_as(C.c_void_p)
+def _addr(a):
+    return a.ctypes.data   # (every caller keeps the array; a c_void_p costs four times as much)
 
 
 class _SysRef:
@@ -174,8 +174,8 @@ class _SysRef:
         self.exps = np.ascontiguousarray(s.exps, dtype=np.uint8)
         self.lo = np.ascontiguousarray(s.box_lo, dtype=np.float64)
         self.hi = np.ascontiguousarray(s.box_hi, dtype=np.float64)
-        self.c = ivs_system(int(s.n_vars), int(s.n_eqs), int(self.off[-1]), _ptr(self.off),
-                            _ptr(self.clo), _ptr(self.chi), _ptr(self.exps))
+        self.c = ivs_system(int(s.n_vars), int(s.n_eqs), int(self.off[-1]), _addr(self.off),
+                            _addr(self.clo), _addr(self.chi), _addr(self.exps))
 
 
 def make_options(tol=1e-6, hs_enable=True, hs_min_depth=0, hs_iters=1, prefilter_fp32=True,
@@ -208,14 +208,14 @@ def result_to_dict(r):
     hi = np.zeros((cnt, n))
     flags = np.zeros(cnt, np.int32)
     depth = np.zeros(cnt, np.int32)
-    _check(lib.ivs_result_boxes(r, _ptr(lo), _ptr(hi), _ptr(flags), _ptr(depth)))
+    _check(lib.ivs_result_boxes(r, _addr(lo), _addr(hi), _addr(flags), _addr(depth)))
     st = ivs_stats()
     _check(lib.ivs_result_stats(r, C.byref(st)))
     stats = {k: getattr(st, k) for k, _ in ivs_stats._fields_}
     db = np.zeros(64, np.int64)
     dk = np.zeros(64, np.int64)
     dh = np.zeros(64, np.int64)
-    _check(lib.ivs_result_depth_stats(r, _ptr(db), _ptr(dk), _ptr(dh)))
+    _check(lib.ivs_result_depth_stats(r, _addr(db), _addr(dk), _addr(dh)))
     stats["depth_boxes"] = db
     stats["depth_kept"] = dk
     stats["depth_hs"] = dh
@@ -232,7 +232,7 @@ def solve(s, box_lo=None, box_hi=None, **opts):
     opts.setdefault("tol", s.tol)
     o = make_options(**opts)
     res = C.c_void_p()
-    rc = lib.ivs_solve(C.byref(ref.c), _ptr(lo), _ptr(hi), C.byref(o), C.byref(res))
+    rc = lib.ivs_solve(C.byref(ref.c), _addr(lo), _addr(hi), C.byref(o), C.byref(res))
     if not res:
         _check(rc)
     try:
@@ -253,8 +253,8 @@ class Plan:
         self.refs = [_SysRef(s) for s in systems]
         self.n_sys = len(systems)
         arr = (ivs_system * self.n_sys)(*[r.c for r in self.refs])
-        los = (C.c_void_p * self.n_sys)(*[_ptr(r.lo) for r in self.refs])
-        his = (C.c_void_p * self.n_sys)(*[_ptr(r.hi) for r in self.refs])
+        los = (C.c_void_p * self.n_sys)(*[_addr(r.lo) for r in self.refs])
+        his = (C.c_void_p * self.n_sys)(*[_addr(r.hi) for r in self.refs])
         if opts is None:
             opts = [make_options(tol=s.tol) for s in systems]
         elif isinstance(opts, dict):
@@ -263,7 +263,7 @@ class Plan:
         cfg = ivs_plan_cfg()
         self._workspace = workspace
         if workspace is not None:
-            cfg.workspace = C.c_void_p(int(workspace.data_ptr()))
+            cfg.workspace = C.c_void_p(int(workspace.data_addr()))
             cfg.workspace_bytes = int(workspace.numel() * workspace.element_size())
         else:
             cfg.workspace_bytes = int(workspace_bytes)
@@ -315,7 +315,7 @@ class Plan:
         boxes to the host."""
         st = ivs_stats()
         db, dk, dh = (np.zeros(64, np.int64) for _ in range(3))
-        _check(self._lib.ivs_plan_depth_stats(self.p, int(s), C.byref(st), _ptr(db), _ptr(dk), _ptr(dh)))
+        _check(self._lib.ivs_plan_depth_stats(self.p, int(s), C.byref(st), _addr(db), _addr(dk), _addr(dh)))
         out = {k: getattr(st, k) for k, _ in ivs_stats._fields_}
         out.update(depth_boxes=db, depth_kept=dk, depth_hs=dh)
         return out
@@ -371,7 +371,7 @@ class Server:
         ref = _SysRef(s)
         o = make_options(**{"tol": s.tol, **opts})
         t = C.c_uint64()
-        _check(self._lib.ivs_server_submit(self.p, C.byref(ref.c), _ptr(ref.lo), _ptr(ref.hi), C.byref(o), C.byref(t)))
+        _check(self._lib.ivs_server_submit(self.p, C.byref(ref.c), _addr(ref.lo), _addr(ref.hi), C.byref(o), C.byref(t)))
         return t.value
 
     def poll(self, ticket):
@@ -419,8 +419,8 @@ def autotune(systems, trial_boxes=200_000, **opts):
     refs = [_SysRef(s) for s in systems]
     n = len(systems)
     arr = (ivs_system * n)(*[r.c for r in refs])
-    los = (C.c_void_p * n)(*[_ptr(r.lo) for r in refs])
-    his = (C.c_void_p * n)(*[_ptr(r.hi) for r in refs])
+    los = (C.c_void_p * n)(*[_addr(r.lo) for r in refs])
+    his = (C.c_void_p * n)(*[_addr(r.hi) for r in refs])
     oarr = (ivs_options * n)(*[make_options(**{"tol": s.tol, **opts}) for s in systems])
     cfg = ivs_plan_cfg()
     rate = C.c_double()
@@ -435,8 +435,8 @@ def solve_batch(systems, **opts):
     refs = [_SysRef(s) for s in systems]
     n = len(systems)
     arr = (ivs_system * n)(*[r.c for r in refs])
-    los = (C.c_void_p * n)(*[_ptr(r.lo) for r in refs])
-    his = (C.c_void_p * n)(*[_ptr(r.hi) for r in refs])
+    los = (C.c_void_p * n)(*[_addr(r.lo) for r in refs])
+    his = (C.c_void_p * n)(*[_addr(r.hi) for r in refs])
     oarr = (ivs_options * n)(*[make_options(**{"tol": s.tol, **opts}) for s in systems])
     outs = (C.c_void_p * n)()
     rc = lib.ivs_solve_batch(n, arr, los, his, oarr, C.sizeof(ivs_options), outs)
@@ -467,8 +467,8 @@ def clusters(lo, hi, with_hulls=True):
     labels = np.zeros(max(k, 1), np.int64)
     hl = np.zeros((max(k, 1), n))
     hh = np.zeros((max(k, 1), n))
-    _check(lib.ivs_clusters(n, k, _ptr(lo), _ptr(hi), C.byref(nc), _ptr(labels),
-                            _ptr(hl) if with_hulls else None, _ptr(hh) if with_hulls else None, k))
+    _check(lib.ivs_clusters(n, k, _addr(lo), _addr(hi), C.byref(nc), _addr(labels),
+                            _addr(hl) if with_hulls else None, _addr(hh) if with_hulls else None, k))
     c = nc.value
     return c, labels[:k], hl[:c], hh[:c]
 
@@ -484,7 +484,7 @@ def clusters_gpu(lo, hi, device=0):
     labels = np.zeros(max(k, 1), np.int64)
     hl = np.zeros((max(k, 1), n))
     hh = np.zeros((max(k, 1), n))
-    _check(lib.ivs_clusters_gpu(n, k, _ptr(lo), _ptr(hi), C.byref(nc), _ptr(labels), _ptr(hl), _ptr(hh), k,
+    _check(lib.ivs_clusters_gpu(n, k, _addr(lo), _addr(hi), C.byref(nc), _addr(labels), _addr(hl), _addr(hh), k,
                                 int(device)))
     c = nc.value
     return c, labels[:k], hl[:c], hh[:c]
@@ -500,7 +500,7 @@ def backtrack_gpu(lo, hi, box_lo, box_hi, level, max_cells=1 << 26, groups=False
     k = lo.shape[0]
     out = C.c_int64()
     grp = C.c_int64()
-    _check(lib.ivs_backtrack_gpu(len(bl), k, _ptr(lo), _ptr(hi), _ptr(bl), _ptr(bh), int(level), int(max_cells),
+    _check(lib.ivs_backtrack_gpu(len(bl), k, _addr(lo), _addr(hi), _addr(bl), _addr(bh), int(level), int(max_cells),
                                  C.byref(out), C.byref(grp), int(device)))
     return (out.value, grp.value) if groups else out.value
 
@@ -517,6 +517,6 @@ def backtrack(lo, hi, box_lo, box_hi, level, max_cells=1 << 26, groups=False):
     k = lo.shape[0]
     out = C.c_int64()
     grp = C.c_int64()
-    _check(lib.ivs_backtrack(len(bl), k, _ptr(lo), _ptr(hi), _ptr(bl), _ptr(bh), int(level), int(max_cells),
+    _check(lib.ivs_backtrack(len(bl), k, _addr(lo), _addr(hi), _addr(bl), _addr(bh), int(level), int(max_cells),
                              C.byref(out), C.byref(grp)))
     return (out.value, grp.value) if groups else out.value

@@ -77,6 +77,11 @@ struct ivs_plan {
     cudaGraphExec_t graph_exec = nullptr;
     int graph_kernels = 0;                 // kernels per sweep of the graph body
     int64_t *h_wave_limit = nullptr;       // pinned
+    // results of the last run, copied in one piece when the first of them is asked for
+    char *h_pack = nullptr;                // pinned: descriptors, then the packed results
+    size_t h_pack_bytes = 0;
+    bool packed = false;
+    std::mutex pack_mu;                    // results of one plan may be read by several threads
     std::vector<double> box_lo_h, box_hi_h;   // initial boxes, n_max per system
 };
 
@@ -130,6 +135,7 @@ void ivs_plan_destroy(ivs_plan *p) {
     if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
     if (p->graph) cudaGraphDestroy(p->graph);
     if (p->h_wave_limit) cudaFreeHost(p->h_wave_limit);
+    if (p->h_pack) cudaFreeHost(p->h_pack);
     if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
     delete p;
 }
@@ -233,6 +239,10 @@ int plan_create_impl(int32_t n_sys, const ivs_system *systems, const double *con
     } else {
         CUDA_TRY(cudaEventCreate(&p->ev0));
         CUDA_TRY(cudaEventCreate(&p->ev1));
+    }
+    if (r && r->h_pack) {
+        std::swap(p->h_pack, r->h_pack);
+        p->h_pack_bytes = r->h_pack_bytes;
     }
     if (r && r->h_ctl) std::swap(p->h_ctl, r->h_ctl);
     else CUDA_TRY(cudaMallocHost((void **)&p->h_ctl, sizeof(WaveCtl)));
@@ -403,6 +413,7 @@ int ivs_plan_run(ivs_plan *p) {
     CUDA_TRY(cudaSetDevice(p->device));
     SweepArgs &a = p->args;
     cudaStream_t st = p->stream;
+    p->packed = false;
     auto t0 = std::chrono::steady_clock::now();
     CUDA_TRY(cudaEventRecord(p->ev0, st));
     CUDA_TRY(cudaMemsetAsync(a.stats, 0, (size_t)p->n_sys * ST_COUNT * sizeof(unsigned long long), st));
@@ -552,6 +563,55 @@ int ivs_plan_stats(ivs_plan *p, ivs_stats *st) {
     return IVS_OK;
 }
 
+// Copies every system's results of the last run into h_pack (one kernel, one copy, one wait);
+// the device side lies in the staging queue, which holds nothing between runs.  False: too
+// large for that (each system is then copied by itself), or a CUDA error.
+static bool pack_results(ivs_plan *p) {
+    std::lock_guard<std::mutex> lk(p->pack_mu);
+    if (p->packed) return true;
+    constexpr size_t kMaxPack = (size_t)16 << 20;
+    const size_t head = align_up((size_t)p->n_sys * sizeof(PackDesc), 256);
+    size_t doubles = 0;
+    for (int s = 0; s < p->n_sys; s++) {
+        const int64_t c = std::min<int64_t>((int64_t)p->h_stats[(size_t)s * ST_COUNT + ST_OUT], p->sys_out_cap[s]);
+        doubles += (size_t)c * (2 * p->sys_n[s] + 1);
+    }
+    const size_t bytes = head + doubles * 8;
+    const DevQueue &q = p->args.stage;   // descriptors in lo, results in mid
+    if (bytes > kMaxPack || head > (size_t)q.cap * 8 || doubles > (size_t)q.cap * p->n_max) return false;
+    if (p->h_pack_bytes < bytes) {
+        if (p->h_pack) cudaFreeHost(p->h_pack);
+        p->h_pack = nullptr;
+        p->h_pack_bytes = 0;
+        const size_t want = align_up(bytes + bytes / 2, 1 << 16);
+        if (cudaMallocHost((void **)&p->h_pack, want) != cudaSuccess) {
+            cudaGetLastError();
+            p->h_pack = nullptr;
+            return false;
+        }
+        p->h_pack_bytes = want;
+    }
+    PackDesc *d = (PackDesc *)p->h_pack;
+    int64_t off = 0;
+    for (int s = 0; s < p->n_sys; s++) {
+        const int64_t c = std::min<int64_t>((int64_t)p->h_stats[(size_t)s * ST_COUNT + ST_OUT], p->sys_out_cap[s]);
+        d[s] = PackDesc{p->sys_out_base[s], c, off, p->sys_n[s]};
+        off += c * (2 * p->sys_n[s] + 1);
+    }
+    if (doubles > 0) {
+        const bool many = p->n_sys > 1;
+        cudaError_t e = cudaSuccess;
+        if (many) e = cudaMemcpyAsync(q.lo, d, (size_t)p->n_sys * sizeof(PackDesc), cudaMemcpyHostToDevice, p->stream);
+        if (e == cudaSuccess)
+            e = launch_pack_results(p->args.out, many ? (const PackDesc *)q.lo : nullptr, d[0], p->n_sys, q.mid, p->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(p->h_pack + head, q.mid, doubles * 8, cudaMemcpyDeviceToHost, p->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
+        if (e != cudaSuccess) return false;   // the per-system copies report it
+    }
+    p->packed = true;
+    return true;
+}
+
 int ivs_plan_result(ivs_plan *p, int32_t s, ivs_result **out) {
     if (!p || !out || s < 0 || s >= p->n_sys) return fail(IVS_ERR_INVALID, "bad arguments");
     *out = nullptr;
@@ -560,10 +620,18 @@ int ivs_plan_result(ivs_plan *p, int32_t s, ivs_result **out) {
     const int64_t total = std::min<int64_t>((int64_t)sv[ST_OUT], p->sys_out_cap[s]);
     const int64_t base = p->sys_out_base[s];
     const int n = p->sys_n[s];
-    std::vector<int32_t> flags(total), depth(total);
-    std::vector<double> lo((size_t)total * n), hi((size_t)total * n);
+    std::unique_ptr<ivs_result> r(new (std::nothrow) ivs_result());
+    if (!r) return fail(IVS_ERR_NOMEM, "host allocation");
+    r->n = n;
     const DevOut &o = p->args.out;
-    if (total > 0) {
+    if (total > 0 && pack_results(p)) {
+        const PackDesc &d = ((const PackDesc *)p->h_pack)[s];
+        const double *lo = (const double *)(p->h_pack + align_up((size_t)p->n_sys * sizeof(PackDesc), 256)) + d.off;
+        const int32_t *flags = (const int32_t *)(lo + 2 * n * total);
+        fill_sorted(r.get(), n, total, lo, lo + n * total, flags, flags + total);
+    } else if (total > 0) {
+        std::vector<int32_t> flags(total), depth(total);
+        std::vector<double> lo((size_t)total * n), hi((size_t)total * n);
         CUDA_TRY(cudaMemcpyAsync(flags.data(), o.flags + base, total * 4, cudaMemcpyDeviceToHost, p->stream));
         CUDA_TRY(cudaMemcpyAsync(depth.data(), o.depth + base, total * 4, cudaMemcpyDeviceToHost, p->stream));
         // coordinate j of entry base + i at j * cap + base + i: one strided copy per array
@@ -572,11 +640,8 @@ int ivs_plan_result(ivs_plan *p, int32_t s, ivs_result **out) {
         CUDA_TRY(cudaMemcpy2DAsync(hi.data(), (size_t)total * 8, o.hi + base, (size_t)o.cap * 8, (size_t)total * 8,
                                    (size_t)n, cudaMemcpyDeviceToHost, p->stream));
         CUDA_TRY(cudaStreamSynchronize(p->stream));
+        fill_sorted(r.get(), n, total, lo, hi, flags, depth);
     }
-    std::unique_ptr<ivs_result> r(new (std::nothrow) ivs_result());
-    if (!r) return fail(IVS_ERR_NOMEM, "host allocation");
-    r->n = n;
-    fill_sorted(r.get(), n, total, lo, hi, flags, depth);
     fill_stats(p, s, &r->st);
     for (int q = 0; q < kDepthSlots; q++) {
         r->depth_boxes[q] = (int64_t)sv[ST_DEPTH_BOXES + q];

@@ -344,6 +344,11 @@ DevOut carve_out(char *base, int64_t cap, int n_max) {
 
 void fill_sorted(ivs_result *r, int n, int64_t total, const std::vector<double> &lo, const std::vector<double> &hi,
                  const std::vector<int32_t> &flags, const std::vector<int32_t> &depth) {
+    fill_sorted(r, n, total, lo.data(), hi.data(), flags.data(), depth.data());
+}
+
+void fill_sorted(ivs_result *r, int n, int64_t total, const double *lo, const double *hi, const int32_t *flags,
+                 const int32_t *depth) {
     r->n = n;
     std::vector<int64_t> idx((size_t)total);
     for (int64_t k = 0; k < total; k++) idx[(size_t)k] = k;

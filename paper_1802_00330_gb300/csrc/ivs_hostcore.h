@@ -26,6 +26,8 @@ namespace host {
 
 // sorts rows given as column-major arrays (lo/hi: n columns of `total` entries) into
 // r's row-major lexicographic order (lo_0, hi_0, lo_1, ...), -0 -> +0
+void fill_sorted(ivs_result *r, int n, int64_t total, const double *lo, const double *hi, const int32_t *flags,
+                 const int32_t *depth);
 void fill_sorted(ivs_result *r, int n, int64_t total, const std::vector<double> &lo, const std::vector<double> &hi,
                  const std::vector<int32_t> &flags, const std::vector<int32_t> &depth);
 

@@ -86,6 +86,15 @@ cudaError_t launch_seed_roots(const SweepArgs &a, const double *d_box_lo, const 
 // serving with regions: empties the regions of the slots with d_cancel[s] != 0 (between
 // sweeps) and lowers the queue total accordingly
 cudaError_t launch_cancel_regions(const SweepArgs &a, const int32_t *d_cancel, cudaStream_t st);
+// One system's results in a packed buffer: n x count lower ends, n x count upper ends
+// (coordinate-major), then count flags and count depths (int32), from `off` (doubles) on.
+struct PackDesc {
+    int64_t base, count, off;
+    int64_t n;
+};
+// packs the results of n_sys systems; desc in device memory, or `one` when n_sys == 1
+cudaError_t launch_pack_results(const DevOut &o, const PackDesc *desc, PackDesc one, int n_sys, double *dst,
+                                cudaStream_t st);
 // appends initial boxes of newly admitted systems (slot ids) on top of the queue, or at
 // the start of each system's region
 cudaError_t launch_admit(const SweepArgs &a, const double *d_lo, const double *d_hi, const int32_t *d_slot,
