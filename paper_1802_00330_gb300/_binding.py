@@ -160,8 +160,15 @@ def _check(rc):
         raise IvsError(rc, f"{lib.ivs_status_str(rc).decode()}: {lib.ivs_last_error().decode()}")
 
 
+def _ptr(a):
+    """A pointer object that holds the array."""
+    return a.ctypes.data_as(C.c_void_p)
+
+
 def _addr(a):
-    return a.ctypes.data   # (every caller keeps the array; a c_void_p costs four times as much)
+    """The array's address, for calls whose caller holds the array (a pointer object costs
+    four times as much, and a call takes about ten of them)."""
+    return a.ctypes.data
 
 
 class _SysRef:
