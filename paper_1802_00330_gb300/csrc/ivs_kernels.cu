@@ -1195,9 +1195,46 @@ cudaError_t configure_eval_kernels(const SweepArgs &a) {
     return allow_max_dynamic_smem((const void *)k_eval64);
 }
 
+// Branches of the contraction stage in a captured sweep.  The kernels of one dimension touch
+// nothing of another's (own survivor list, own part of a.cand, own cursors; results, staging
+// and counters through atomics), and most sweeps of a batch leave the small dimensions a few
+// boxes each, whose 25-50 us of latency added up one dimension after the other (96-system
+// batch of n = 2..5: 3.7 of 5.3 ms; the call 8.0 -> 6.7 ms, 24 served requests 70 -> 67 ms, the
+// 64-system batch 257 -> 252).  Branch 0 is the capturing stream; the largest dimensions
+// get a branch of their own, the rest share them in reverse order.
+constexpr int kBranches = 4;
+struct Branches {
+    cudaStream_t st[kBranches] = {};
+    cudaEvent_t fork = nullptr, join[kBranches] = {};
+    int n = 1;
+    cudaError_t open(cudaStream_t main, int dims) {
+        st[0] = main;
+        n = dims < kBranches ? dims : kBranches;
+        cudaError_t e = cudaSuccess;
+        if (n > 1) e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+        for (int b = 1; b < n && e == cudaSuccess; b++) {
+            e = cudaStreamCreateWithFlags(&st[b], cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[b], cudaEventDisableTiming);
+        }
+        return e;
+    }
+    // branch of the q-th largest of the dimensions
+    int of(int q) const {
+        const int r = q % (2 * n);
+        return r < n ? r : 2 * n - 1 - r;
+    }
+    ~Branches() {
+        for (int b = 1; b < kBranches; b++) {
+            if (st[b]) cudaStreamDestroy(st[b]);
+            if (join[b]) cudaEventDestroy(join[b]);
+        }
+        if (fork) cudaEventDestroy(fork);
+    }
+};
+
 static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int n_hs_dims, int eval_blocks,
                                      int num_sms, cudaStream_t st, cudaEvent_t *ev, cudaGraphConditionalHandle h,
-                                     int use_cond, int *kernels) {
+                                     int use_cond, int *kernels, const Branches *br = nullptr) {
     int count = 4;   // wave_begin, eval, eval64, commit
     // ev (optional): n_hs_dims + 5 events recorded between the stages
     const size_t head = a.single ? (size_t)a.head_smem : 0;
@@ -1208,6 +1245,22 @@ static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int
     if (ev) cudaEventRecord(ev[2], st);
     k_eval64<<<num_sms * 4, kEval64Threads, head, st>>>(a);
     if (ev) cudaEventRecord(ev[3], st);
+    if (br && br->n > 1) {
+        cudaError_t e = cudaEventRecord(br->fork, st);
+        for (int b = 1; b < br->n && e == cudaSuccess; b++) e = cudaStreamWaitEvent(br->st[b], br->fork, 0);
+        for (int q = 0; q < n_hs_dims && e == cudaSuccess; q++) {
+            int kq = 0;
+            e = launch_hs(a, hs_dims[n_hs_dims - 1 - q], num_sms, br->st[br->of(q)], &kq);
+            count += kq;
+        }
+        // (joined also after an error, so that the capture can end)
+        for (int b = 1; b < br->n; b++) {
+            cudaError_t je = cudaEventRecord(br->join[b], br->st[b]);
+            if (je == cudaSuccess) je = cudaStreamWaitEvent(st, br->join[b], 0);
+            if (e == cudaSuccess) e = je;
+        }
+        if (e != cudaSuccess) return e;
+    } else
     for (int q = 0; q < n_hs_dims; q++) {
         int kq = 0;
         cudaError_t e = launch_hs(a, hs_dims[q], num_sms, st, &kq);
@@ -1245,13 +1298,15 @@ cudaError_t build_sweep_graph(const SweepArgs &a, const int *hs_dims, int n_hs_d
     if (e == cudaSuccess) e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp);
     cudaStream_t cs = nullptr;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
+    Branches br;
+    if (e == cudaSuccess) e = br.open(cs, n_hs_dims);
     if (e == cudaSuccess) {
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             (void)eval_threads;
             cudaError_t le = launch_sweep_impl(a, hs_dims, n_hs_dims, eval_blocks, num_sms, cs, nullptr, h, 1,
-                                               kernels_per_sweep);
+                                               kernels_per_sweep, &br);
             cudaGraph_t captured = nullptr;
             e = cudaStreamEndCapture(cs, &captured);
             if (e == cudaSuccess && le != cudaSuccess) e = le;
