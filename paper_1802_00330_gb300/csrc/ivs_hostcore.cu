@@ -142,7 +142,8 @@ void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
         }
     }
     const int CX = (int)cix.size();
-    const BlobLayout L = blob_layout(T, P, F, TF, E, CX);
+    const int SC = T;
+    const BlobLayout L = blob_layout(T, P, F, TF, E, CX, SC);
     const size_t off = h.blobs.size();
     h.blobs.resize(off + L.bytes, 0);
     char *base = h.blobs.data() + off;
@@ -178,6 +179,7 @@ void pack_blob(HostTables &h, const SysBuild &b, DevSys &d, int n_fterms) {
     d.n_fterms = TF;
     d.n_tv = E;
     d.n_cix = CX;
+    d.n_scr = SC;
     d.blob_bytes = (int32_t)L.bytes;
     d.head_bytes = (int32_t)L.head;
 }

@@ -76,6 +76,7 @@ struct DevSys {
     uint8_t eq_order[kMaxVars];   // equations by number of terms (when m <= kMaxVars)
     int32_t krawczyk;      // 1: Krawczyk contraction (eq 15-16) instead of Gauss-Seidel
     int32_t bisect;        // 1: widest-coordinate bisection (2 children) instead of 2^n
+    int32_t n_scr;         // the screen's term records (n_terms, or 0)
     int32_t head_bytes;    // bytes of the blob's head (ivs_tab.cuh)
     int32_t gap_split;     // 1: two boxes at an extended-division gap (Gauss-Seidel only)
 };

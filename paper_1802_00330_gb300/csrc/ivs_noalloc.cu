@@ -39,7 +39,7 @@ static __device__ __align__(256) unsigned char g_scratch[kScratch];
 
 std::mutex g_mu;                        // serialises host-side set-up and the static buffers
 void *g_scratch_addr[kMaxDevices] = {};
-alignas(16) char g_host_blob[kMaxBlob]; // compiled term table staged on the host
+alignas(16) char g_host_blob[kMaxBlob + 32]; // compiled term table staged on the host (its parts are padded)
 WaveCtl g_ctl;                          // host copy of the sweep control block
 char *g_errbuf = nullptr;               // the current call's message buffer (caller's)
 int32_t g_errlen = 0;
@@ -100,7 +100,7 @@ bool pack_static(const ivs_system *s, DevSys &d) {
     }, [&]() { P++; });
     if (T > kMaxTerms) return false;
     const BlobLayout L = blob_layout(T, P, F);
-    if (L.bytes > kMaxBlob) return false;
+    if (((L.fac + (uint32_t)F + 4 + 15u) & ~15u) > kMaxBlob) return false;   // the table proper
     std::memset(g_host_blob, 0, L.bytes);
     int t = 0, p = 0, f = 0;
     int32_t *poly_off = reinterpret_cast<int32_t *>(g_host_blob + L.poly_off);

@@ -34,7 +34,7 @@ using Clock = std::chrono::steady_clock;
 
 namespace {
 
-constexpr uint32_t kBlobSlot = 128 * 1024;   // term-table bytes per slot (n = 12, 14 terms of degree 4
+constexpr uint32_t kBlobSlot = 240 * 1024, kBlobTable = 128 * 1024;   // term-table bytes per slot (n = 12, 14 terms of degree 4
                                              // per equation need about 50 KB)
 
 struct Request {
@@ -315,7 +315,8 @@ int ivs_server::step(std::vector<std::pair<uint64_t, ivs_result *>> &finished) {
         const ivs_system sv = rq.view();
         compile_system(h, &sv, &rq.opt);
         DevSys d = h.sys[0];
-        if ((uint32_t)d.blob_bytes > kBlobSlot) {
+        // the screen's records and the child index have room of their own in a slot
+        if ((int64_t)d.blob_bytes - 16ll * d.n_scr - d.n_cix > kBlobTable || (uint32_t)d.blob_bytes > kBlobSlot) {
             ivs_result *r = new (std::nothrow) ivs_result();
             if (r) { r->status = IVS_ERR_INVALID; r->n = rq.n; }
             finished.push_back({rq.ticket, r});

@@ -19,18 +19,19 @@
 namespace ivs {
 
 // byte layout of a system blob with T terms, P polynomials, F factors, TF terms in the
-// equations F_i, E term-combination entries and CX child-index entries
+// equations F_i, E term-combination entries, CX child-index entries and SC screen records
+// (T, or 0 where the system is never screened)
 struct BlobLayout {
     uint32_t cs, scr, clo, chi, clo32, chi32, poly_off, tinfo, fac, head, tv_off, tv_map, cix, bytes;
 };
 // The head (all that evaluates polynomials) comes first: kernels that do not read the
 // per-parent tables cache the head alone (at n = 8 5 KB of 45, a third block per SM for k_hs<8>
 // and k_screen<8> in plans of one system).
-__host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 0, int E = 0, int CX = 0) {
+__host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 0, int E = 0, int CX = 0, int SC = 0) {
     BlobLayout L;
     uint32_t o = 0;
     L.cs = o;        o += 16u * T;
-    L.scr = o;       o += 16u * T;
+    L.scr = o;       o += 16u * SC;
     L.clo = o;       o += 8u * T;
     L.chi = o;       o += 8u * T;
     L.clo32 = o;     o += 4u * T;
@@ -85,7 +86,7 @@ struct SysTab {
 };
 
 __device__ __forceinline__ SysTab make_tab(const char *blob, const DevSys &S) {
-    const BlobLayout L = blob_layout(S.n_terms, S.n_polys, S.n_facs, S.n_fterms, S.n_tv, S.n_cix);
+    const BlobLayout L = blob_layout(S.n_terms, S.n_polys, S.n_facs, S.n_fterms, S.n_tv, S.n_cix, S.n_scr);
     SysTab t;
     t.cs = reinterpret_cast<const float4 *>(blob + L.cs);
     t.scr = reinterpret_cast<const ScrTerm *>(blob + L.scr);
