@@ -132,7 +132,7 @@ TRAFFIC = {
     ("batched", "hs_n8"): {"sources_sha256": "c44aac276b43290460c0650e3d9a0e8ae810783df0d16dae8a9dc0db22b76c93",
                            "bytes_per_hs_box": 57.46, "default_options_only": True, "wave_children": 1 << 24},
 }
-KERNEL_SOURCES = ("ivs_hs.cuh", "ivs_tab.cuh", "ivs_interval.cuh", "ivs_internal.h", "ivs_kernels.cuh")
+KERNEL_SOURCES = ("ivs_hs.cuh", "ivs_screen.cuh", "ivs_div.cuh", "ivs_tab.cuh", "ivs_interval.cuh", "ivs_internal.h", "ivs_kernels.cuh")
 
 
 def _code_only(text):
@@ -381,14 +381,17 @@ def _timed_runs(plan, stream, flush, steps):
 
 def class_rooflines(B, prof, systems, krawczyk, fp64_rate, fp32_rate, ktimes, steps):
     """Per kernel class: algorithmic operations of the work it did over its CUDA-event
-    time, against the measured directed rate of its pipe.  hs_n<k>: hs_ops of every sweep
-    run on the systems of size k; eval (FP32 stage): one natural-form evaluation per
+    time, against the measured directed rate of its pipe.  hs_n<k>: hs_ops of the sweeps
+    on the systems of size k that FP64 has to run -- from four variables on those that
+    shrink their box (or find no preconditioner), since an FP32 screen decides the others in
+    the sweeps it takes: a lower bound; eval (FP32 stage): one natural-form evaluation per
     child; eval64: one FP64 evaluation per undecided child."""
     per = [prof.result_stats(k) for k in range(len(systems))]
     ops, hs_boxes = {}, {}
     for s, st in zip(systems, per):
         key = f"hs_n{s.n_vars}"
-        ops[key] = ops.get(key, 0.0) + st["hs_applied"] * hs_ops(s, krawczyk)
+        swept = st["hs_applied"] if s.n_vars < 4 else st["hs_contracted"] + st["hs_singular"]
+        ops[key] = ops.get(key, 0.0) + swept * hs_ops(s, krawczyk)
         hs_boxes[key] = hs_boxes.get(key, 0) + int(st["depth_hs"].sum())
         ops["eval"] = ops.get("eval", 0.0) + st["boxes"] * eval_ops(s)
         ops["eval64"] = ops.get("eval64", 0.0) + st["eval64_boxes"] * eval_ops(s)

@@ -34,6 +34,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include "ivs_div.cuh"
 #include "ivs_internal.h"
 #include "ivs_interval.cuh"
 #include "ivs_kernels.cuh"
@@ -245,7 +246,7 @@ __device__ __forceinline__ void gj_block(double *sd, int *si, int t) {
             const int j = e / BB, b = e % BB;
             if (!run[b] || bad[b]) continue;
             const double pv = sd[C::PIV + b];
-            G[(k * N + j) * BB + b] = __ddiv_rn(j == k ? 1.0 : G[(k * N + j) * BB + b], pv);
+            G[(k * N + j) * BB + b] = div_exact<DIV_RN>(j == k ? 1.0 : G[(k * N + j) * BB + b], pv);
         }
         __syncthreads();
         // elimination of column k from the other rows (eq 24): one row per unit, or one
@@ -473,12 +474,12 @@ __device__ __forceinline__ void gs_block(double *sd, int *si, int t, GapRec &gr)
                 xc = sd[C::XC + i * BB + b];
                 ivd pc[2];
                 if (up) {   // upper quotient; lower ends of the pieces x_i - pc
-                    np = extdiv_pieces(kind, 0.0, __ddiv_ru(xd.un, xd.ud), pc);
+                    np = extdiv_pieces(kind, 0.0, div_exact<DIV_RU>(xd.un, xd.ud), pc);
 #pragma unroll
                     for (int q = 0; q < 2; q++)
                         if (q < np) SX[q * BB + b] = __dsub_rd(xc, pc[q].hi);
                 } else {    // lower quotient; upper ends
-                    np = extdiv_pieces(kind, __ddiv_rd(xd.ln, xd.ld), 0.0, pc);
+                    np = extdiv_pieces(kind, div_exact<DIV_RD>(xd.ln, xd.ld), 0.0, pc);
 #pragma unroll
                     for (int q = 0; q < 2; q++)
                         if (q < np) yhi[q] = __dsub_ru(xc, pc[q].lo);
