@@ -439,7 +439,8 @@ int ivs_plan_run(ivs_plan *p) {
             CUDA_TRY(cudaMemcpyAsync(p->h_stats.data(), a.stats, p->h_stats.size() * sizeof(unsigned long long),
                                      cudaMemcpyDeviceToHost, st));
             CUDA_TRY(cudaStreamSynchronize(st));
-            p->launches += (int64_t)p->graph_kernels * (p->h_ctl->waves - waves_done);
+            // (plans of one system: and the pop in front of the loop)
+            p->launches += (int64_t)p->graph_kernels * (p->h_ctl->waves - waves_done) + (a.single ? 1 : 0);
             waves_done = p->h_ctl->waves;
             if (p->h_ctl->error) { status = IVS_ERR_NOMEM; break; }
             if (p->h_ctl->top == 0) break;

@@ -128,6 +128,8 @@ struct WaveCtl {
     int64_t out_count;      // accepted boxes written
     int32_t cursor;         // evaluation kernel's parent cursor
     int32_t error;          // sticky: 1 = queue full
+    int32_t ticket;         // k_commit's blocks that have read the sweep's bounds
+    int32_t pad_;
     int64_t surv_count[kMaxVars + 1];   // survivors per n (index n)
     int64_t hs_cursor[kMaxVars + 1];    // Hansen-Sengupta kernels' work cursors
     int64_t screen_cursor[kMaxVars + 1];   // the FP32 screen's work cursors

@@ -195,6 +195,35 @@ __device__ __forceinline__ int64_t parent_index(const SweepArgs &a, int64_t base
     return a.rg.base[lo] + a.rg.rem[lo] + (p - a.rg.prefix[lo]);
 }
 
+// One system: every entry has the fan-out F = 2^n (2 when bisected) except the initial box
+// (fan-out 1, alone in the queue when popped), so the pop is a closed form.
+__device__ __forceinline__ void begin_single(const SweepArgs &a, WaveCtl *c, int64_t top, bool root) {
+    int64_t k = 0, children = 0;
+    if (top > 0) {
+        if (root) {
+            k = 1;
+            children = 1;
+        } else {
+            const int64_t F = fan_out(a.tb.sys[0], 0u);
+            k = a.wave_children / F;
+            const int64_t by_room = (a.q.cap - top) / (F - 1);
+            k = k < by_room ? k : by_room;
+            k = k < top ? k : top;
+            children = k * F;
+        }
+    }
+    if (k <= 0 && top > 0) c->error = 1;
+    c->base = top - k;
+    c->k = k;
+    c->children = children;
+    c->cursor = 0;
+    c->staged = 0;
+    reset_lists(c);
+    c->cand_count = 0;
+    c->cand_cursor = 0;
+    c->waves += 1;
+}
+
 __global__ void __launch_bounds__(kBeginThreads) k_wave_begin(SweepArgs a) {
     // log2 children of the window's entries; serving: the sort keys of the slots
     extern __shared__ __align__(8) unsigned char s_fan[];
@@ -208,33 +237,7 @@ __global__ void __launch_bounds__(kBeginThreads) k_wave_begin(SweepArgs a) {
     const int64_t top = c->top;
     const int t = threadIdx.x;
     if (a.single) {
-        // one system: every entry has fan-out F = 2^n except the initial box (fan-out 1,
-        // alone in the queue when popped), so the scan below reduces to a closed form
-        if (t != 0) return;
-        int64_t k = 0, children = 0;
-        if (top > 0) {
-            if (a.q.meta[top - 1] & kRootFlag) {
-                k = 1;
-                children = 1;
-            } else {
-                const int64_t F = fan_out(a.tb.sys[0], 0u);
-                k = a.wave_children / F;
-                const int64_t by_room = (a.q.cap - top) / (F - 1);
-                k = k < by_room ? k : by_room;
-                k = k < top ? k : top;
-                children = k * F;
-            }
-        }
-        if (k <= 0 && top > 0) c->error = 1;
-        c->base = top - k;
-        c->k = k;
-        c->children = children;
-        c->cursor = 0;
-        c->staged = 0;
-        reset_lists(c);
-        c->cand_count = 0;
-        c->cand_cursor = 0;
-        c->waves += 1;
+        if (t == 0) begin_single(a, c, top, top > 0 && (a.q.meta[top - 1] & kRootFlag) != 0);
         return;
     }
     const int64_t window = top < (int64_t)kBeginThreads * kBeginPer ? top : (int64_t)kBeginThreads * kBeginPer;
@@ -298,14 +301,31 @@ __global__ void __launch_bounds__(kBeginThreads) k_wave_begin(SweepArgs a) {
     c->waves += 1;
 }
 
-// Moves the sweep's new parents onto the queue.  In the sweep graph (use_cond) block 0
-// also sets the WHILE condition: more sweeps while the queue is non-empty after this
-// commit, no error occurred and the sweep limit is not reached (nothing after the commit
-// changes any of them).
+// Moves the sweep's new parents onto the queue.  In the sweep graph (use_cond) it also sets
+// the WHILE condition: more sweeps while the queue is non-empty after this commit, no error
+// occurred and the sweep limit is not reached (nothing after the commit changes any of
+// them).  use_cond 2 (plans of one system): when there are more, the last block that has
+// read this sweep's bounds also pops the next sweep's parents, a closed form that reads no
+// queue entry, so the sweep needs no k_wave_begin of its own (n = 5 bisection, 35 sweeps: 2217 ->
+// 2173 us; n = 6 plan: 1081 -> 1070).
 __global__ void k_commit(SweepArgs a, int n_max, cudaGraphConditionalHandle h, int use_cond) {
-    const WaveCtl *c = a.ctl;
+    WaveCtl *c = a.ctl;
     const int64_t staged = c->staged, base = c->base;
-    if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) {
+    if (use_cond == 2) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (atomicAdd(&c->ticket, 1) == (int)gridDim.x - 1) {
+                __threadfence();
+                const int64_t top = base + staged;
+                const bool more = top > 0 && c->error == 0 && c->waves < c->wave_limit;
+                c->ticket = 0;
+                c->top = top;
+                if (more) begin_single(a, c, top, false);
+                cudaGraphSetConditional(h, more ? 1u : 0u);
+            }
+        }
+    } else if (use_cond && blockIdx.x == 0 && threadIdx.x == 0) {
         const bool more = base + staged > 0 && c->error == 0 && c->waves < c->wave_limit;
         cudaGraphSetConditional(h, more ? 1u : 0u);
     }
@@ -324,7 +344,7 @@ __global__ void k_commit(SweepArgs a, int n_max, cudaGraphConditionalHandle h, i
         a.q.sys[d] = a.stage.sys[i];
         a.q.meta[d] = a.stage.meta[i];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->top = base + staged;
+    if (use_cond != 2 && blockIdx.x == 0 && threadIdx.x == 0) c->top = base + staged;
 }
 
 __global__ void k_seed_roots(SweepArgs a, const double *box_lo, const double *box_hi,
@@ -348,6 +368,7 @@ __global__ void k_seed_roots(SweepArgs a, const double *box_lo, const double *bo
         c->out_count = 0;
         c->cursor = 0;
         c->error = 0;
+        c->ticket = 0;
         c->waves = 0;
         c->cand_count = 0;
         c->cand_cursor = 0;
@@ -1235,11 +1256,11 @@ struct Branches {
 static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int n_hs_dims, int eval_blocks,
                                      int num_sms, cudaStream_t st, cudaEvent_t *ev, cudaGraphConditionalHandle h,
                                      int use_cond, int *kernels, const Branches *br = nullptr) {
-    int count = 4;   // wave_begin, eval, eval64, commit
+    int count = use_cond == 2 ? 3 : 4;   // (wave_begin,) eval, eval64, commit
     // ev (optional): n_hs_dims + 5 events recorded between the stages
     const size_t head = a.single ? (size_t)a.head_smem : 0;
     if (ev) cudaEventRecord(ev[0], st);
-    k_wave_begin<<<1, kBeginThreads, kBeginSmem, st>>>(a);
+    if (use_cond != 2) k_wave_begin<<<1, kBeginThreads, kBeginSmem, st>>>(a);
     if (ev) cudaEventRecord(ev[1], st);
     k_eval<<<eval_blocks, kEvalThreads, eval_smem_bytes(a), st>>>(a);
     if (ev) cudaEventRecord(ev[2], st);
@@ -1268,7 +1289,7 @@ static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int
         count += kq;
         if (ev) cudaEventRecord(ev[4 + q], st);
     }
-    k_commit<<<num_sms * 4, 256, 0, st>>>(a, a.max_fan_shift, h, use_cond);
+    k_commit<<<num_sms * (use_cond == 2 ? 2 : 4), 256, 0, st>>>(a, a.max_fan_shift, h, use_cond);
     if (ev) cudaEventRecord(ev[4 + n_hs_dims], st);
     if (kernels) *kernels = count;
     return cudaGetLastError();
@@ -1294,8 +1315,21 @@ cudaError_t build_sweep_graph(const SweepArgs &a, const int *hs_dims, int n_hs_d
     cp.conditional.handle = h;
     cp.conditional.type = cudaGraphCondTypeWhile;
     cp.conditional.size = 1;
-    cudaGraphNode_t node;
-    if (e == cudaSuccess) e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp);
+    // plans of one system: the first sweep's pop in front of the loop, the others in k_commit
+    const bool fused = a.single && a.rg.n == 0;
+    cudaGraphNode_t node, first = nullptr;
+    if (e == cudaSuccess && fused) {
+        SweepArgs copy = a;
+        void *args[1] = {&copy};
+        cudaKernelNodeParams kp = {};
+        kp.func = (void *)k_wave_begin;
+        kp.gridDim = dim3(1);
+        kp.blockDim = dim3(kBeginThreads);
+        kp.sharedMemBytes = (unsigned)kBeginSmem;
+        kp.kernelParams = args;
+        e = cudaGraphAddKernelNode(&first, g, nullptr, 0, &kp);
+    }
+    if (e == cudaSuccess) e = cudaGraphAddNode(&node, g, fused ? &first : nullptr, nullptr, fused ? 1 : 0, &cp);
     cudaStream_t cs = nullptr;
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     Branches br;
@@ -1305,7 +1339,7 @@ cudaError_t build_sweep_graph(const SweepArgs &a, const int *hs_dims, int n_hs_d
         e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
             (void)eval_threads;
-            cudaError_t le = launch_sweep_impl(a, hs_dims, n_hs_dims, eval_blocks, num_sms, cs, nullptr, h, 1,
+            cudaError_t le = launch_sweep_impl(a, hs_dims, n_hs_dims, eval_blocks, num_sms, cs, nullptr, h, fused ? 2 : 1,
                                                kernels_per_sweep, &br);
             cudaGraph_t captured = nullptr;
             e = cudaStreamEndCapture(cs, &captured);
