@@ -57,6 +57,43 @@ struct Key {
 };
 __device__ __forceinline__ bool key_less(Key x, Key y) { return x.a < y.a || (x.a == y.a && x.b < y.b); }
 
+// Device memory of one call, given back at its end.  Small buffers share blocks of 16 MB: an
+// allocation and its release cost ~20 us, and a call takes a dozen (2e4 boxes of 9 variables: 2.8
+// -> 2.4 ms).
+struct Scratch {
+    static constexpr size_t kBlock = (size_t)16 << 20;
+    std::vector<void *> v;
+    char *cur = nullptr;
+    size_t left = 0;
+    ~Scratch() {
+        for (void *p : v) cudaFree(p);
+    }
+    template <class T>
+    cudaError_t get(T **p, size_t n) {
+        const size_t bytes = (std::max<size_t>(n, 1) * sizeof(T) + 255) & ~(size_t)255;
+        *p = nullptr;
+        if (bytes > left && bytes < kBlock / 4) {
+            void *q = nullptr;
+            cudaError_t e = cudaMalloc(&q, kBlock);
+            if (e != cudaSuccess) return e;
+            v.push_back(q);
+            cur = (char *)q;
+            left = kBlock;
+        }
+        if (bytes <= left) {
+            *p = (T *)cur;
+            cur += bytes;
+            left -= bytes;
+            return cudaSuccess;
+        }
+        void *q = nullptr;
+        cudaError_t e = cudaMalloc(&q, bytes);
+        if (e == cudaSuccess) v.push_back(q);
+        *p = (T *)q;
+        return e;
+    }
+};
+
 // ---- scan (exclusive, int64) -------------------------------------------------------------
 constexpr int kScanThreads = 1024;
 
@@ -84,14 +121,12 @@ __global__ void k_scan_add(int64_t *out, int64_t count, const int64_t *offs) {
 
 // exclusive scan of count values; *total (device) receives their sum
 cudaError_t scan_exclusive(const int64_t *in, int64_t *out, int64_t count, int64_t *total, cudaStream_t st,
-                           std::vector<void *> &scratch) {
+                           Scratch &scratch) {
     if (count <= 0) return cudaMemsetAsync(total, 0, sizeof(int64_t), st);
     const int64_t nb = (count + kScanThreads - 1) / kScanThreads;
     int64_t *sums = nullptr, *offs = nullptr;
-    cudaError_t e = cudaMalloc(&sums, (size_t)nb * sizeof(int64_t));
-    if (e == cudaSuccess) scratch.push_back(sums);
-    if (e == cudaSuccess) e = cudaMalloc(&offs, (size_t)nb * sizeof(int64_t));
-    if (e == cudaSuccess) scratch.push_back(offs);
+    cudaError_t e = scratch.get(&sums, (size_t)nb);
+    if (e == cudaSuccess) e = scratch.get(&offs, (size_t)nb);
     if (e != cudaSuccess) return e;
     k_scan_blocks<<<(unsigned)nb, kScanThreads, 0, st>>>(in, out, count, sums);
     if (nb == 1) return cudaMemcpyAsync(total, sums, sizeof(int64_t), cudaMemcpyDeviceToDevice, st);
@@ -103,9 +138,10 @@ cudaError_t scan_exclusive(const int64_t *in, int64_t *out, int64_t count, int64
 
 // ---- bitonic sort of 128-bit keys ----------------------------------------------------------
 // 2^18 keys: 0.44 -> 0.31 ms a sort.  Every thread of a step holds a pair (element index from
-// the pair index), blocks of 2048 keys sort in shared memory, and a global pass does two
+// the pair index), blocks of 1024 keys sort in shared memory (2048 made
+// sets of a few thousand boxes 0.1 ms slower), and a global pass does two
 // steps on four keys per thread, so a merge of 2^18 keys reads the keys 4 times, not 8.
-constexpr int kSortBlock = 2048;     // elements per shared-memory stage
+constexpr int kSortBlock = 1024;     // elements per shared-memory stage
 constexpr int kSortThreads = kSortBlock / 2;
 
 // element x of a pair / quad with its partner at distance j: bit log2(j) of the index is 0
@@ -285,7 +321,7 @@ __global__ void __launch_bounds__(kUniteWarps * 32) k_unite(const K *key, int64_
         constexpr int J = N > 1 ? 1 : 0;   // the coordinate tested first
         const K *kl = key + (int64_t)(2 * J) * count, *kh = key + (int64_t)(2 * J + 1) * count;
         int held = 0;   // pairs in the warp's queue
-        for (int64_t q = p0 + 1 + warp; q < last; q += kUniteWarps) {
+        for (int64_t q = p0 + 1 + blockIdx.y * kUniteWarps + warp; q < last; q += kUniteWarps * gridDim.y) {
             bool touch = kl[q] <= h[J] && l[J] <= kh[q] && q > p && q < stop;
             if (!__any_sync(0xFFFFFFFFu, touch)) continue;
 #pragma unroll
@@ -310,7 +346,9 @@ __global__ void __launch_bounds__(kUniteWarps * 32) k_unite(const K *key, int64_
 template <class K>
 cudaError_t launch_unite(int n, const K *key, int64_t count, const int64_t *end, const Key *id, int64_t *par, int *err,
                          cudaStream_t st) {
-    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>((count + 31) / 32, 1 << 20));
+    // small sets: the ranges are split over more blocks, so that the chip has a few per SM
+    const unsigned gx = (unsigned)std::max<int64_t>(1, std::min<int64_t>((count + 31) / 32, 1 << 20));
+    const dim3 grid(gx, (unsigned)std::max<int64_t>(1, std::min<int64_t>(32, 2432 / (int64_t)gx)));
     switch (n) {
 #define IVS_UNITE(N) case N: k_unite<K, N><<<grid, kUniteWarps * 32, 0, st>>>(key, count, end, id, par, err); break;
         IVS_UNITE(1) IVS_UNITE(2) IVS_UNITE(3) IVS_UNITE(4) IVS_UNITE(5) IVS_UNITE(6) IVS_UNITE(7) IVS_UNITE(8)
@@ -564,21 +602,6 @@ __global__ void k_cl_hull_out(const unsigned long long *hlo, const unsigned long
 }
 
 // ---- host drivers -----------------------------------------------------------------------------
-struct Scratch {
-    std::vector<void *> v;
-    ~Scratch() {
-        for (void *p : v) cudaFree(p);
-    }
-    template <class T>
-    cudaError_t get(T **p, size_t n) {
-        void *q = nullptr;
-        cudaError_t e = cudaMalloc(&q, std::max<size_t>(n, 1) * sizeof(T));
-        if (e == cudaSuccess) v.push_back(q);
-        *p = (T *)q;
-        return e;
-    }
-};
-
 unsigned grid_for(int64_t n) { return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 152 * 32)); }
 
 #define RT_TRY(x)                                                                                   \
@@ -622,7 +645,7 @@ int backtrack_device(const BoxView &v, const double *box_lo, const double *box_h
     RT_TRY(cudaMemsetAsync(flags, 0, 2 * sizeof(int), st));
     k_bt_count<<<grid_for(v.count), 256, 0, st>>>(v, g, max_cells, m, range, flags);
     RT_TRY(cudaGetLastError());
-    RT_TRY(scan_exclusive(m, offs, v.count, tot, st, sc.v));
+    RT_TRY(scan_exclusive(m, offs, v.count, tot, st, sc));
     int64_t total = 0;
     int hf[2] = {0, 0};
     RT_TRY(cudaMemcpyAsync(&total, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
@@ -640,7 +663,7 @@ int backtrack_device(const BoxView &v, const double *box_lo, const double *box_h
     RT_TRY(sc.get(&fl, total));
     RT_TRY(sc.get(&pos, total));
     k_flag_distinct<<<grid_for(total), 256, 0, st>>>(keys, total, fl);
-    RT_TRY(scan_exclusive(fl, pos, total, tot, st, sc.v));
+    RT_TRY(scan_exclusive(fl, pos, total, tot, st, sc));
     int64_t d = 0;
     RT_TRY(cudaMemcpyAsync(&d, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     RT_TRY(sc.get(&uniq, total));
@@ -718,7 +741,7 @@ int clusters_device(const BoxView &v, int64_t *n_clusters, int64_t *label_h, dou
     RT_TRY(sc.get(&num, v.count));
     RT_TRY(sc.get(&tot, 1));
     k_cl_first<<<grid_for(v.count), 256, 0, st>>>(par, v.count, work);
-    RT_TRY(scan_exclusive(work, num, v.count, tot, st, sc.v));
+    RT_TRY(scan_exclusive(work, num, v.count, tot, st, sc));
     int64_t nc = 0;
     int he = 0;
     RT_TRY(cudaMemcpyAsync(&nc, tot, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
