@@ -270,7 +270,7 @@ class Plan:
         cfg = ivs_plan_cfg()
         self._workspace = workspace
         if workspace is not None:
-            cfg.workspace = C.c_void_p(int(workspace.data_addr()))
+            cfg.workspace = C.c_void_p(int(workspace.data_ptr()))
             cfg.workspace_bytes = int(workspace.numel() * workspace.element_size())
         else:
             cfg.workspace_bytes = int(workspace_bytes)
