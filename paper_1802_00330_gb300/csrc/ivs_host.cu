@@ -191,6 +191,7 @@ int plan_create_impl(int32_t n_sys, const ivs_system *systems, const double *con
         (void)0;
         h.sys.back().shadow = (o->prefilter_fp32 && std::getenv("IVS_NO_SHADOW") == nullptr &&
                                shadow_safe(&systems[s], box_lo[s], box_hi[s])) ? 1 : 0;
+        h.sys.back().scr_tiny = screen_tiny(&systems[s], box_lo[s], box_hi[s]);
         if (o->time_budget_s > 0)
             p->time_budget_s = p->time_budget_s > 0 ? std::min(p->time_budget_s, o->time_budget_s) : o->time_budget_s;
     }

@@ -239,6 +239,36 @@ bool shadow_safe(const ivs_system *s, const double *lo, const double *hi) {
     return true;
 }
 
+// The FP32 screen forms a term of degree g in at most 2 g + 2 roundings to nearest (powers,
+// products, the coefficient's own).  One whose result is subnormal loses up to 2^-150 beside
+// its relative 2^-24, and what multiplies it later -- the coefficient and powers, in either
+// order -- is at most B = max(|c|, 1) prod max(|x_j|, 1)^e_j, with |c| 15 times larger in a
+// derivative.  The sum over an equation's terms of 15 (2 g + 2) 2^-150 B, taken 2.1 times or
+// more as 2^-144 (g + 1) B, bounds it for F_i and every J_ij.  Terms of ordinary size add
+// nothing to the 1e-30 that every radius has anyway; with B = 1e28 the radii grow to 1e-14
+// and boxes whose values are that small stay open (monomials of 2^-144 under coefficients of
+// 2^92 were taken for 0 before).
+float screen_tiny(const ivs_system *s, const double *lo, const double *hi) {
+    const int n = s->n_vars;
+    double top = 0.0;
+    for (int i = 0; i < s->n_eqs; i++) {
+        double sum = 0.0;
+        for (int t = s->eq_offsets[i]; t < s->eq_offsets[i + 1]; t++) {
+            double b = std::max({std::fabs(s->coef_lo[t]), std::fabs(s->coef_hi ? s->coef_hi[t] : s->coef_lo[t]), 1.0});
+            int g = 0;
+            for (int j = 0; j < n; j++) {
+                const int a = s->exps[(size_t)t * n + j];
+                const double m = std::max({std::fabs(lo[j]), std::fabs(hi[j]), 1.0});
+                g += a;
+                for (int q = 0; q < a; q++) b *= m;
+            }
+            sum += (g + 1) * b;
+        }
+        top = std::max(top, sum);
+    }
+    return to_float_up((double)kScrTiny + std::ldexp(top, -144));
+}
+
 void compile_system(HostTables &h, const ivs_system *s, const ivs_options *o) {
     const int n = s->n_vars, m = s->n_eqs;
     SysBuild bld;

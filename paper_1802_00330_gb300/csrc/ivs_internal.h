@@ -78,6 +78,7 @@ struct DevSys {
     int32_t bisect;        // 1: widest-coordinate bisection (2 children) instead of 2^n
     int32_t n_scr;         // the screen's term records (n_terms, or 0)
     int32_t head_bytes;    // bytes of the blob's head (ivs_tab.cuh)
+    float scr_tiny;        // the screen: what underflow may add to a polynomial's float value
     int32_t gap_split;     // 1: two boxes at an extended-division gap (Gauss-Seidel only)
 };
 

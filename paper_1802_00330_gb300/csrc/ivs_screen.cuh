@@ -57,7 +57,7 @@ namespace ivs {
 namespace scr {
 constexpr unsigned kFull = 0xFFFFFFFFu;
 constexpr float kU = 5.9604645e-8f;     // 2^-24, the float rounding unit
-constexpr float kTiny = 1e-30f;         // absolute part of every radius (underflow)
+constexpr float kTiny = kScrTiny;       // absolute part of every radius (underflow)
 constexpr float kHuge = 1e15f;          // larger magnitudes are left to FP64
 constexpr float kSlack = 1.0f + 1e-5f;  // relative part of the final comparisons
 
@@ -131,13 +131,15 @@ __device__ __forceinline__ void pow32(float l, float h, float m, int k, float &a
 
 // Natural extension of polynomial p over the box (ends xl, xh, stride 32 floats).  The FP64
 // ends are real interval arithmetic up to rounding, so the float ends differ from them by at
-// most (operations + input roundings) x 2^-24 x the sum of the terms' magnitudes.
+// most (operations + input roundings) x 2^-24 x the sum of the terms' magnitudes, plus what
+// products lose below float's normal range: tiny, a bound over the system's initial box
+// (host::screen_tiny).  Magnitudes that underflow themselves are covered by it too.
 // Terms of up to three factors of degree up to kScrPow read the box's powers (pl, ph: computed
 // once per box, stride 32) and one 16-byte record; the others go through the term table.
 // (With the table alone every term decoded its factors and raised its powers again; with that, the
 // n = 11 stage 30.3 -> 23.6 ms and kinema 93.6 -> 87.4, the pivot search by trees included.)
 __device__ __forceinline__ Poly poly_c(const SysTab &T, int p, const float *xl, const float *xh, const float *pl_,
-                                       const float *ph_) {
+                                       const float *ph_, float tiny) {
     const int t0 = T.poly_off[p], t1 = T.poly_off[p + 1];
     const float nt = (float)(t1 - t0 + 6);
     float lo = 0.0f, hi = 0.0f, rad = 0.0f;
@@ -204,13 +206,13 @@ __device__ __forceinline__ Poly poly_c(const SysTab &T, int p, const float *xl, 
         rad += fmaxf(fabsf(ce.x), fabsf(ce.w)) * pm * ((float)(2 * deg) + nt);
     }
     // a single constant that float holds exactly has no error
-    return Poly{0.5f * (lo + hi), 0.5f * (hi - lo), (exact ? 0.0f : rad * (1.01f * kU)) + kTiny};
+    return Poly{0.5f * (lo + hi), 0.5f * (hi - lo), exact ? kTiny : rad * (1.01f * kU) + tiny};
 }
 
 // value of polynomial p at the box's centre (each coordinate within 2 units of the largest
 // end's magnitude), with its radius
 __device__ __forceinline__ float2 poly_v(const SysTab &T, int p, const float *xl, const float *xh, const float *pl_,
-                                         const float *ph_, const float *px_) {
+                                         const float *ph_, const float *px_, float tiny) {
     const int t0 = T.poly_off[p], t1 = T.poly_off[p + 1];
     const float nt = (float)(t1 - t0 + 6);
     float v = 0.0f, w = 0.0f, rad = 0.0f;
@@ -247,7 +249,7 @@ __device__ __forceinline__ float2 poly_v(const SysTab &T, int p, const float *xl
         if (!(info & kTermPoint)) w += (ce.w - ce.x) * pm;
         rad += fmaxf(fabsf(ce.x), fabsf(ce.w)) * pm * ((float)(4 * deg) + nt);
     }
-    return make_float2(v, fmaf(rad, 1.01f * kU, w * 1.01f) + kTiny);
+    return make_float2(v, fmaf(rad, 1.01f * kU, w * 1.01f) + tiny);
 }
 
 __device__ __forceinline__ float mul_ru(float a, float b) { return __fmul_ru(a, b); }
@@ -401,13 +403,13 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
             for (int q = warp; q < N * N + N; q += NT / 32) {
                 if (!on) continue;
                 if (q < N * N) {
-                    const Poly v = poly_c(T, S.j_poly + q, xl, xh, sf + C::PL + b, sf + C::PH + b);
+                    const Poly v = poly_c(T, S.j_poly + q, xl, xh, sf + C::PL + b, sf + C::PH + b, S.scr_tiny);
                     sf[C::JC + q * P + b] = v.c;
                     sf[C::JW + q * P + b] = v.w;
                     sf[C::JR + q * P + b] = v.r;
                 } else {
                     const float2 v = poly_v(T, S.f_poly + (q - N * N), xl, xh, sf + C::PL + b, sf + C::PH + b,
-                                            sf + C::PX + b);
+                                            sf + C::PX + b, S.scr_tiny);
                     sf[C::FV + (q - N * N) * BB + b] = v.x;
                     sf[C::FR + (q - N * N) * BB + b] = v.y;
                 }

@@ -325,6 +325,7 @@ int ivs_server::step(std::vector<std::pair<uint64_t, ivs_result *>> &finished) {
             continue;
         }
         d.shadow = (rq.opt.prefilter_fp32 && shadow_safe(&sv, rq.lo.data(), rq.hi.data())) ? 1 : 0;
+        d.scr_tiny = screen_tiny(&sv, rq.lo.data(), rq.hi.data());
         d.blob_off = (int64_t)s * kBlobSlot;
         d.out_base = (int64_t)s * rps;
         d.out_cap = rq.opt.max_results > 0 ? std::min<int64_t>(rq.opt.max_results, rps) : rps;

@@ -66,6 +66,7 @@ __host__ __device__ inline uint32_t term_info(uint32_t start, uint32_t cnt, doub
 // (more factors, higher exponents or a coefficient interval: the term table is read), 1
 // simple, 3 simple, constant and exact in float.
 constexpr int kScrPow = 3;
+constexpr float kScrTiny = 1e-30f;   // the least absolute error that the screen allows a polynomial's value
 struct ScrTerm {
     float c, w;
     uint32_t fac, kind;
