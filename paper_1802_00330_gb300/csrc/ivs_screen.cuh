@@ -442,7 +442,8 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
                 const float err = (rv + fr + 1e-5f * (av + fabsf(f))) * kSlack;
                 if (!(av < kHuge && fabsf(f) < kHuge)) atomicOr(&s_bad[b], 1);
                 else if (fabsf(f) > av + err) atomicOr(&s_fate[b], 1);     // excluded
-                else if (!(fabsf(f) + err <= av)) atomicOr(&s_fate[b], 2);   // open
+                // (av holds J's ends moved out by the radii; they may lie as far in)
+                else if (!(fabsf(f) + err + rv * kSlack <= av)) atomicOr(&s_fate[b], 2);   // open
             }
         }
         __syncthreads();
