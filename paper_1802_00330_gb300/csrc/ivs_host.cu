@@ -321,10 +321,15 @@ int plan_create_impl(int32_t n_sys, const ivs_system *systems, const double *con
                                  cudaMemcpyHostToDevice, p->stream));
     a.tb.sys = (const DevSys *)p->tables_mem;
     a.tb.blobs = (const char *)p->tables_mem + sys_bytes;
-    // one system: every kernel caches its blob in shared memory (if it fits)
-    a.single = (n_sys == 1 && h.sys[0].blob_bytes <= 48 * 1024) ? 1 : 0;
-    a.blob_smem = a.single ? h.sys[0].blob_bytes : 0;
-    a.head_smem = a.single ? h.sys[0].head_bytes : 0;
+    // One system: k_eval caches its blob in shared memory, the other kernels the blob's head, each
+    // up to 48 KB.  From n = 9 on the per-parent tables make the blob larger than that while the
+    // head stays at 15-32 KB, and k_eval reads such a blob through L1 (with its head cached the
+    // same times: n = 11 part 27.0 ms either way).  Head cached and pop in k_commit against neither: n = 10 part
+    // 3.39 -> 3.29 ms, n = 11 27.3 -> 27.1, n = 12 21.4 -> 21.2.
+    constexpr int kCache = 48 * 1024;
+    a.single = n_sys == 1 ? 1 : 0;
+    a.blob_smem = a.single && h.sys[0].blob_bytes <= kCache ? h.sys[0].blob_bytes : 0;
+    a.head_smem = a.single && h.sys[0].head_bytes <= kCache ? h.sys[0].head_bytes : 0;
     choose_eval_layout(a, h.sys.data(), n_sys);
     if (std::getenv("IVS_NO_COMBO")) {   // per-child evaluation instead of tables
         a.tv_entries = 0;

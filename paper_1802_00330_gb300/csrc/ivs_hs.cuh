@@ -902,8 +902,8 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     using D = hsd::Cfg<N, kNarrowBoxes>;
     *kernels = 2;
     // cache the term table in shared memory when the plan holds one system and it fits
-    const bool cache = a.single && (size_t)a.head_smem + C::BYTES <= kHsSmemLimit;
-    const bool ncache = a.single && (size_t)a.head_smem + D::BYTES <= kHsSmemLimit;
+    const bool cache = a.head_smem && (size_t)a.head_smem + C::BYTES <= kHsSmemLimit;
+    const bool ncache = a.head_smem && (size_t)a.head_smem + D::BYTES <= kHsSmemLimit;
     const size_t smem = (cache ? (size_t)a.head_smem : 0) + C::BYTES;
     const size_t nsmem = (ncache ? (size_t)a.head_smem : 0) + D::BYTES;
     int per_sm = 0, n_per_sm = 0;   // blocks per SM at these shared memory sizes
@@ -920,7 +920,7 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     if constexpr (N >= kScreenMinVars) {
       if (a.screen) {
         using S = scr::Cfg<N>;
-        const bool scache = a.single && (size_t)a.head_smem + S::BYTES <= kScreenSmemLimit;
+        const bool scache = a.head_smem && (size_t)a.head_smem + S::BYTES <= kScreenSmemLimit;
         const size_t ssmem = (scache ? (size_t)a.head_smem : 0) + S::BYTES;
         e = allow_max_dynamic_smem((const void *)k_screen<N>);
         if (e != cudaSuccess) return e;

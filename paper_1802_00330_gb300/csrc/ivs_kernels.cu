@@ -922,7 +922,7 @@ __device__ __forceinline__ void eval_warp(const SweepArgs &a, WaveCtl *ctl, cons
     const uint32_t meta = a.q.meta[pi];
     const DevSys S = a.tb.sys[sys];
     if (block_form(a, S)) return;   // the block pass takes it
-    const SysTab T = make_tab(a.single ? s_blob : a.tb.blobs + S.blob_off, S);
+    const SysTab T = make_tab(a.blob_smem ? s_blob : a.tb.blobs + S.blob_off, S);
     const bool root = (meta & kRootFlag) != 0;
     const int depth = (int)(meta & kDepthMask) + (root ? 0 : 1);
     if (sys != w.sys || depth != w.depth || S.max_boxes > 0) {
@@ -972,7 +972,7 @@ __device__ __forceinline__ void eval_block(const SweepArgs &a, WaveCtl *ctl, con
     const int sys = a.q.sys[pi];
     const uint32_t meta = a.q.meta[pi];
     const DevSys S = a.tb.sys[sys];
-    const SysTab T = make_tab(a.single ? s_blob : a.tb.blobs + S.blob_off, S);
+    const SysTab T = make_tab(a.blob_smem ? s_blob : a.tb.blobs + S.blob_off, S);
     const bool root = (meta & kRootFlag) != 0;
     const int depth = (int)(meta & kDepthMask) + (root ? 0 : 1);
     if (t == 0) *s_flag = over_budget(a, sys, S) ? 1 : 0;
@@ -1013,7 +1013,7 @@ __device__ __forceinline__ void eval_block(const SweepArgs &a, WaveCtl *ctl, con
 // asks for a block.
 __global__ void __launch_bounds__(kEvalThreads, 3) k_eval(SweepArgs a) {
     extern __shared__ __align__(16) char s_blob[];
-    float4 *s_tv = reinterpret_cast<float4 *>(s_blob + (a.single ? a.blob_smem : 0));
+    float4 *s_tv = reinterpret_cast<float4 *>(s_blob + a.blob_smem);
     __shared__ double s_p[kEvalWarps][3][kMaxVars];
     __shared__ float s_f[kEvalWarps][4][kMaxVars];
     __shared__ float s_e[kEvalWarps][6][kMaxVars];
@@ -1029,9 +1029,8 @@ __global__ void __launch_bounds__(kEvalThreads, 3) k_eval(SweepArgs a) {
     // blocks beyond what K parents need leave at once (the others take every parent), so
     // a small sweep does not pay for the whole grid
     if (block_pass ? (int64_t)blockIdx.x >= K : (int64_t)blockIdx.x * kEvalWarps >= K) return;
-    if (a.single) {
-        const DevSys &S0 = a.tb.sys[0];
-        copy_blob(s_blob, a.tb.blobs + S0.blob_off, (uint32_t)S0.blob_bytes);
+    if (a.blob_smem) {
+        copy_blob(s_blob, a.tb.blobs + a.tb.sys[0].blob_off, (uint32_t)a.blob_smem);
         __syncthreads();
     }
     if (warp_pass) {
@@ -1093,9 +1092,8 @@ __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
     const bool split = count <= kSplitCandidates;
     // not needed for this many candidates
     if ((int64_t)blockIdx.x * blockDim.x >= (split ? 8 * count : count)) return;
-    if (a.single) {
-        const DevSys &S0 = a.tb.sys[0];
-        copy_blob(s_blob, a.tb.blobs + S0.blob_off, (uint32_t)S0.head_bytes);
+    if (a.head_smem) {
+        copy_blob(s_blob, a.tb.blobs + a.tb.sys[0].blob_off, (uint32_t)a.head_smem);
         __syncthreads();
     }
     const unsigned lane = lane_id();
@@ -1116,7 +1114,7 @@ __global__ void __launch_bounds__(kEval64Threads) k_eval64(SweepArgs a) {
             const int64_t pi = sv.parent;
             sys = a.q.sys[pi];
             const DevSys S = a.tb.sys[sys];
-            const SysTab Tb = make_tab(a.single ? s_blob : a.tb.blobs + S.blob_off, S);
+            const SysTab Tb = make_tab(a.head_smem ? s_blob : a.tb.blobs + S.blob_off, S);
             n = S.n;
             for (int j = 0; j < n; j++) {
                 const bool up = (sv.child >> j) & 1u;
@@ -1191,7 +1189,7 @@ static cudaError_t launch_hs(const SweepArgs &a, int n, int num_sms, cudaStream_
 }
 
 size_t eval_smem_bytes(const SweepArgs &a) {
-    return (size_t)(a.single ? a.blob_smem : 0) + (size_t)a.tv_entries * sizeof(float4);
+    return (size_t)a.blob_smem + (size_t)a.tv_entries * sizeof(float4);
 }
 
 cudaError_t allow_max_dynamic_smem(const void *func) {
@@ -1258,7 +1256,7 @@ static cudaError_t launch_sweep_impl(const SweepArgs &a, const int *hs_dims, int
                                      int use_cond, int *kernels, const Branches *br = nullptr) {
     int count = use_cond == 2 ? 3 : 4;   // (wave_begin,) eval, eval64, commit
     // ev (optional): n_hs_dims + 5 events recorded between the stages
-    const size_t head = a.single ? (size_t)a.head_smem : 0;
+    const size_t head = (size_t)a.head_smem;
     if (ev) cudaEventRecord(ev[0], st);
     if (use_cond != 2) k_wave_begin<<<1, kBeginThreads, kBeginSmem, st>>>(a);
     if (ev) cudaEventRecord(ev[1], st);

@@ -33,9 +33,9 @@ struct SweepArgs {
     int64_t wave_children;       // children a sweep may evaluate
     int32_t max_fan_shift;       // max n over the plan's systems
     int32_t n_sys;
-    int32_t single;              // 1: one system; kernels cache its blob in shared memory
-    int32_t blob_smem;           // bytes of that blob
-    int32_t head_smem;           // bytes of its head, all that the contraction's kernels cache
+    int32_t single;              // 1: one system (closed-form pop, in k_commit after the first sweep)
+    int32_t blob_smem;           // bytes of its blob when k_eval caches it in shared memory, else 0
+    int32_t head_smem;           // bytes of the blob's head when the other kernels cache it, else 0
     int32_t tv_entries;          // table entries of a block of k_eval (0: no tables)
     int32_t eval_forms;          // bit 0: some system's parents go to warps, bit 1: to blocks;
                                  // bit 2: every parent has few children (a warp also in narrow sweeps)
