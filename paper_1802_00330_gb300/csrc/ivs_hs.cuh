@@ -896,21 +896,37 @@ constexpr size_t kHsSmemLimit = 227 * 1024 - 64;
 // the screen's dynamic shared memory, less its static arrays
 constexpr size_t kScreenSmemLimit = 220 * 1024;
 
+// Blocks per SM of a kernel with *smem bytes of its own; *cache and *smem with the head's bytes added
+// when it fits the limit and leaves as many blocks.
+inline cudaError_t cached_occupancy(const void *func, int threads, int head, size_t limit, size_t *smem, int *per_sm,
+                                    bool *cache) {
+    int with = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, func, threads, *smem);
+    if (e != cudaSuccess || head <= 0 || *smem + (size_t)head > limit) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&with, func, threads, *smem + (size_t)head);
+    if (e == cudaSuccess && with >= *per_sm) {
+        *cache = true;
+        *smem += (size_t)head;
+    }
+    return e;
+}
+
 template <int N>
 static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st, int *kernels) {
     using C = hsd::Cfg<N, kWideBoxes<N>>;
     using D = hsd::Cfg<N, kNarrowBoxes>;
     *kernels = 2;
-    // cache the term table in shared memory when the plan holds one system and it fits
-    const bool cache = a.head_smem && (size_t)a.head_smem + C::BYTES <= kHsSmemLimit;
-    const bool ncache = a.head_smem && (size_t)a.head_smem + D::BYTES <= kHsSmemLimit;
-    const size_t smem = (cache ? (size_t)a.head_smem : 0) + C::BYTES;
-    const size_t nsmem = (ncache ? (size_t)a.head_smem : 0) + D::BYTES;
+    // The kernels cache the head of the term table in shared memory when the plan holds one system,
+    // it fits and no resident block is lost for it: k_hs<8> runs 2 blocks per SM with the
+    // recipes' head and 3 without (n = 8 plan 7.82 -> 7.70 ms), k_hs<10> 1 and 2 (n = 10 part 11.66 -> 11.53).
+    size_t smem = C::BYTES, nsmem = D::BYTES;
     int per_sm = 0, n_per_sm = 0;   // blocks per SM at these shared memory sizes
+    bool cache = false, ncache = false;
     cudaError_t e = allow_max_dynamic_smem((const void *)k_hs<N>);
     if (e == cudaSuccess) e = allow_max_dynamic_smem((const void *)k_hs_narrow<N>);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_hs<N>, C::NT, smem);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n_per_sm, k_hs_narrow<N>, D::NT, nsmem);
+    if (e == cudaSuccess) e = cached_occupancy((const void *)k_hs<N>, C::NT, a.head_smem, kHsSmemLimit, &smem, &per_sm, &cache);
+    if (e == cudaSuccess)
+        e = cached_occupancy((const void *)k_hs_narrow<N>, D::NT, a.head_smem, kHsSmemLimit, &nsmem, &n_per_sm, &ncache);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
     if (n_per_sm < 1) n_per_sm = 1;
@@ -920,12 +936,12 @@ static cudaError_t launch_hs_n(const SweepArgs &a, int num_sms, cudaStream_t st,
     if constexpr (N >= kScreenMinVars) {
       if (a.screen) {
         using S = scr::Cfg<N>;
-        const bool scache = a.head_smem && (size_t)a.head_smem + S::BYTES <= kScreenSmemLimit;
-        const size_t ssmem = (scache ? (size_t)a.head_smem : 0) + S::BYTES;
-        e = allow_max_dynamic_smem((const void *)k_screen<N>);
-        if (e != cudaSuccess) return e;
+        size_t ssmem = S::BYTES;
         int s_per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&s_per_sm, k_screen<N>, S::NT, ssmem);
+        bool scache = false;
+        e = allow_max_dynamic_smem((const void *)k_screen<N>);
+        if (e == cudaSuccess)
+            e = cached_occupancy((const void *)k_screen<N>, S::NT, a.head_smem, kScreenSmemLimit, &ssmem, &s_per_sm, &scache);
         if (e != cudaSuccess) return e;
         k_screen<N><<<num_sms * (s_per_sm < 1 ? 1 : s_per_sm), S::NT, ssmem, st>>>(a, scache ? 1 : 0, screen_min);
         e = cudaGetLastError();

@@ -25,8 +25,7 @@ struct BlobLayout {
     uint32_t cs, scr, clo, chi, clo32, chi32, poly_off, tinfo, fac, head, tv_off, tv_map, cix, bytes;
 };
 // The head (all that evaluates polynomials) comes first: kernels that do not read the
-// per-parent tables cache the head alone (at n = 8 5 KB of 45, a third block per SM for k_hs<8>
-// and k_screen<8> in plans of one system).
+// per-parent tables cache the head alone (at n = 8 11 KB of 28).
 __host__ __device__ inline BlobLayout blob_layout(int T, int P, int F, int TF = 0, int E = 0, int CX = 0, int SC = 0) {
     BlobLayout L;
     uint32_t o = 0;
