@@ -2,8 +2,8 @@
 //
 // The library's division runs on the FP64 pipe, which is the contraction's bottleneck: 1000
 // cycles in a dependent chain and 7 (to nearest) to 12 (directed) adds' worth of its rate,
-// against 361 cycles of the integer and FP32 pipes here (equal on 1.7e9 quotients in the three
-// roundings).  Contraction stage: n = 5 bisection 1.58 -> 1.47 ms, n = 6 solve 0.74 -> 0.71,
+// against 361 cycles of the integer and FP32 pipes here (a test compares 2.3e8 pairs of
+// operands with the library in the three roundings).  Contraction stage: n = 5 bisection 1.58 -> 1.47 ms, n = 6 solve 0.74 -> 0.71,
 // kinema 87.9 -> 84.1, n = 8 of the 64-system batch 128.8 -> 123.6.  2n
 // divisions follow one another in a box's sweep.  This one is a digit recurrence of very high
 // radix (Ercegovac and Lang, Division and Square Root, 1994): signed digits of 17-18 bits,
@@ -32,9 +32,13 @@ __device__ __forceinline__ double div_library(double a, double b) {
 }
 
 __device__ __forceinline__ float rcp_approx(float x) {
+#ifdef __CUDA_ARCH__
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
+#else
+    return 1.0f / x;   // compiled for the host by a test
+#endif
 }
 
 // a / b rounded to nearest even (DIV_RN), down (DIV_RD) or up (DIV_RU): the library's value for
@@ -57,15 +61,16 @@ __device__ __forceinline__ double div_exact(double a, double b) {
         r <<= 1;
         e -= 1;
     }
-    // scale: remainder / 2^23 and divisor / 2^21 as floats, digits of 2^18, 2^17, 2^17
+    // scale: remainder / 2^23 and divisor / 2^21 as floats, digits of 2^18, 2^17, 2^17.  The products
+    // reach 2^72 and their differences stay below 2^53, so they are taken modulo 2^64.
     const float inv = rcp_approx(__uint2float_rn((uint32_t)(mb >> 21))) * 0x1p+20f;   // 2^(23 - 21 + 18)
     const int d1 = __float2int_rn(__int2float_rn((int)(r >> 23)) * inv);
-    r = (int64_t)((uint64_t)r << 18) - (int64_t)d1 * mb;
+    r = (int64_t)(((uint64_t)r << 18) - (uint64_t)(int64_t)d1 * (uint64_t)mb);
     const float inv2 = inv * 0.5f;
     const int d2 = __float2int_rn(__int2float_rn((int)(r >> 23)) * inv2);
-    r = (int64_t)((uint64_t)r << 17) - (int64_t)d2 * mb;
+    r = (int64_t)(((uint64_t)r << 17) - (uint64_t)(int64_t)d2 * (uint64_t)mb);
     const int d3 = __float2int_rn(__int2float_rn((int)(r >> 23)) * inv2);
-    r = (int64_t)((uint64_t)r << 17) - (int64_t)d3 * mb;
+    r = (int64_t)(((uint64_t)r << 17) - (uint64_t)(int64_t)d3 * (uint64_t)mb);
     int64_t q = ((((int64_t)d1 << 17) + d2) << 17) + d3;
     if (r < 0) {
         q -= 1;
