@@ -304,16 +304,13 @@ __device__ __forceinline__ shv sh_mul(shv x, shv y, bool &poison) {
                                      lyh ? y.hd : y.ld, lyh ? y.hu : y.lu, lyh ? syh : syl);
     const float2 h1 = enc_mul_signed(uxh ? x.hd : x.ld, uxh ? x.hu : x.lu, uxh ? sxh : sxl,
                                      uyh ? y.hd : y.ld, uyh ? y.hu : y.lu, uyh ? syh : syl);
-    // the second pair only when some lane of the warp has both operands straddling 0 (for
-    // the other lanes it repeats the first pair); a box's halves meet at 0 on these grids, so
-    // it is rare
-    if (__any_sync(__activemask(), ss)) {
-        const float2 l2 = enc_mul_signed(ss ? x.hd : (lxh ? x.hd : x.ld), ss ? x.hu : (lxh ? x.hu : x.lu),
-                                         ss ? sxh : (lxh ? sxh : sxl), ss ? y.ld : (lyh ? y.hd : y.ld),
-                                         ss ? y.lu : (lyh ? y.hu : y.lu), ss ? syl : (lyh ? syh : syl));
-        const float2 h2 = enc_mul_signed(ss ? x.hd : (uxh ? x.hd : x.ld), ss ? x.hu : (uxh ? x.hu : x.lu),
-                                         ss ? sxh : (uxh ? sxh : sxl), ss ? y.hd : (uyh ? y.hd : y.ld),
-                                         ss ? y.hu : (uyh ? y.hu : y.lu), ss ? syh : (uyh ? syh : syl));
+    // the second pair only where both operands straddle 0 (elsewhere it would repeat the first
+    // pair); a box's halves meet at 0 on these grids, so it is rare.  Each lane branches by
+    // itself: the callers' loops diverge, so a vote of the lanes that happen to be together
+    // would say nothing
+    if (ss) {
+        const float2 l2 = enc_mul_signed(x.hd, x.hu, sxh, y.ld, y.lu, syl);
+        const float2 h2 = enc_mul_signed(x.hd, x.hu, sxh, y.hd, y.hu, syh);
         return {fminf(l1.x, l2.x), fminf(l1.y, l2.y), fmaxf(h1.x, h2.x), fmaxf(h1.y, h2.y)};
     }
     return {l1.x, l1.y, h1.x, h1.y};
