@@ -80,7 +80,7 @@ struct ivs_plan {
     // results of the last run, copied in one piece when the first of them is asked for
     char *h_pack = nullptr;                // pinned: descriptors, then the packed results
     size_t h_pack_bytes = 0;
-    bool packed = false;
+    int packed = 0;                        // 0 not asked for yet, 1 there, -1 not to be had this way
     std::mutex pack_mu;                    // results of one plan may be read by several threads
     std::vector<double> box_lo_h, box_hi_h;   // initial boxes, n_max per system
 };
@@ -419,7 +419,7 @@ int ivs_plan_run(ivs_plan *p) {
     CUDA_TRY(cudaSetDevice(p->device));
     SweepArgs &a = p->args;
     cudaStream_t st = p->stream;
-    p->packed = false;
+    p->packed = 0;
     auto t0 = std::chrono::steady_clock::now();
     CUDA_TRY(cudaEventRecord(p->ev0, st));
     CUDA_TRY(cudaMemsetAsync(a.stats, 0, (size_t)p->n_sys * ST_COUNT * sizeof(unsigned long long), st));
@@ -572,16 +572,22 @@ int ivs_plan_stats(ivs_plan *p, ivs_stats *st) {
 
 // Copies every system's results of the last run into h_pack (one kernel, one copy, one wait);
 // the device side lies in the staging queue, which holds nothing between runs.  False: too
-// large for that (each system is then copied by itself), or a CUDA error.
+// large for that (each system is then copied by itself), or a CUDA error; a run's first call
+// decides.
 static bool pack_results(ivs_plan *p) {
     std::lock_guard<std::mutex> lk(p->pack_mu);
-    if (p->packed) return true;
+    if (p->packed) return p->packed > 0;
+    p->packed = -1;
     constexpr size_t kMaxPack = (size_t)16 << 20;
     const size_t head = align_up((size_t)p->n_sys * sizeof(PackDesc), 256);
+    auto rows = [&](int s) {
+        return std::min<int64_t>((int64_t)p->h_stats[(size_t)s * ST_COUNT + ST_OUT], p->sys_out_cap[s]);
+    };
     size_t doubles = 0;
+    int64_t most = 0;
     for (int s = 0; s < p->n_sys; s++) {
-        const int64_t c = std::min<int64_t>((int64_t)p->h_stats[(size_t)s * ST_COUNT + ST_OUT], p->sys_out_cap[s]);
-        doubles += (size_t)c * (2 * p->sys_n[s] + 1);
+        doubles += (size_t)rows(s) * (2 * p->sys_n[s] + 1);
+        most = std::max(most, rows(s));
     }
     const size_t bytes = head + doubles * 8;
     const DevQueue &q = p->args.stage;   // descriptors in lo, results in mid
@@ -601,21 +607,21 @@ static bool pack_results(ivs_plan *p) {
     PackDesc *d = (PackDesc *)p->h_pack;
     int64_t off = 0;
     for (int s = 0; s < p->n_sys; s++) {
-        const int64_t c = std::min<int64_t>((int64_t)p->h_stats[(size_t)s * ST_COUNT + ST_OUT], p->sys_out_cap[s]);
-        d[s] = PackDesc{p->sys_out_base[s], c, off, p->sys_n[s]};
-        off += c * (2 * p->sys_n[s] + 1);
+        d[s] = PackDesc{p->sys_out_base[s], rows(s), off, p->sys_n[s]};
+        off += rows(s) * (2 * p->sys_n[s] + 1);
     }
     if (doubles > 0) {
         const bool many = p->n_sys > 1;
         cudaError_t e = cudaSuccess;
         if (many) e = cudaMemcpyAsync(q.lo, d, (size_t)p->n_sys * sizeof(PackDesc), cudaMemcpyHostToDevice, p->stream);
         if (e == cudaSuccess)
-            e = launch_pack_results(p->args.out, many ? (const PackDesc *)q.lo : nullptr, d[0], p->n_sys, q.mid, p->stream);
+            e = launch_pack_results(p->args.out, many ? (const PackDesc *)q.lo : nullptr, d[0], p->n_sys, most, q.mid,
+                                    p->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(p->h_pack + head, q.mid, doubles * 8, cudaMemcpyDeviceToHost, p->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
         if (e != cudaSuccess) return false;   // the per-system copies report it
     }
-    p->packed = true;
+    p->packed = 1;
     return true;
 }
 

@@ -92,8 +92,8 @@ struct PackDesc {
     int64_t base, count, off;
     int64_t n;
 };
-// packs the results of n_sys systems; desc in device memory, or `one` when n_sys == 1
-cudaError_t launch_pack_results(const DevOut &o, const PackDesc *desc, PackDesc one, int n_sys, double *dst,
+// packs the results of n_sys systems, at most `most` of one; desc in device memory, or `one` when n_sys == 1
+cudaError_t launch_pack_results(const DevOut &o, const PackDesc *desc, PackDesc one, int n_sys, int64_t most, double *dst,
                                 cudaStream_t st);
 // appends initial boxes of newly admitted systems (slot ids) on top of the queue, or at
 // the start of each system's region
