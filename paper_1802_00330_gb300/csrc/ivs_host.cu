@@ -189,9 +189,8 @@ int plan_create_impl(int32_t n_sys, const ivs_system *systems, const double *con
             p->dims.push_back(systems[s].n_vars);
         compile_system(h, &systems[s], o);
         (void)0;
-        h.sys.back().shadow = (o->prefilter_fp32 && std::getenv("IVS_NO_SHADOW") == nullptr &&
-                               shadow_safe(&systems[s], box_lo[s], box_hi[s])) ? 1 : 0;
-        h.sys.back().scr_tiny = screen_tiny(&systems[s], box_lo[s], box_hi[s]);
+        const bool in_range = float_range(&systems[s], box_lo[s], box_hi[s], &h.sys.back().scr_tiny);
+        h.sys.back().shadow = (o->prefilter_fp32 && std::getenv("IVS_NO_SHADOW") == nullptr && in_range) ? 1 : 0;
         if (o->time_budget_s > 0)
             p->time_budget_s = p->time_budget_s > 0 ? std::min(p->time_budget_s, o->time_budget_s) : o->time_budget_s;
     }

@@ -215,31 +215,11 @@ int validate(const ivs_system *s, const double *lo, const double *hi, const ivs_
     return IVS_OK;
 }
 
-// F_i and J_ij polynomials of one system appended to the tables.  J_ij = sum over terms t
-// of equation i with a_tj > 0 of [down(c_lo a_tj), up(c_hi a_tj)] x^(a_t - e_j), in term
-// order; its factors keep the variable order of the term.
+// Two properties of the system on its initial box, in one pass over its terms.
 // The FP32 shadow may decide boxes only when no FP32 intermediate can overflow: every
 // term's magnitude over the initial box, times the number of terms, stays below 1e30
 // (float max ~3.4e38).  Otherwise the plain FP32 prefilter (sound under overflow) runs.
-bool shadow_safe(const ivs_system *s, const double *lo, const double *hi) {
-    const int n = s->n_vars;
-    for (int i = 0; i < s->n_eqs; i++) {
-        const int nt = s->eq_offsets[i + 1] - s->eq_offsets[i];
-        for (int t = s->eq_offsets[i]; t < s->eq_offsets[i + 1]; t++) {
-            double c = std::max(std::fabs(s->coef_lo[t]), std::fabs(s->coef_hi ? s->coef_hi[t] : s->coef_lo[t]));
-            double b = c;
-            for (int j = 0; j < n; j++) {
-                const int a = s->exps[(size_t)t * n + j];
-                const double m = std::max(std::fabs(lo[j]), std::fabs(hi[j]));
-                for (int q = 0; q < a; q++) b *= std::max(m, 1.0);
-            }
-            if (!(b * (nt + 1) < 1e30)) return false;
-        }
-    }
-    return true;
-}
-
-// The FP32 screen forms a term of degree g in at most 2 g + 2 roundings to nearest (powers,
+// scr_tiny: the FP32 screen forms a term of degree g in at most 2 g + 2 roundings to nearest (powers,
 // products, the coefficient's own).  One whose result is subnormal loses up to 2^-150 beside
 // its relative 2^-24, and what multiplies it later -- the coefficient and powers, in either
 // order -- is at most B = max(|c|, 1) prod max(|x_j|, 1)^e_j, with |c| 15 times larger in a
@@ -248,27 +228,38 @@ bool shadow_safe(const ivs_system *s, const double *lo, const double *hi) {
 // nothing to the 1e-30 that every radius has anyway; with B = 1e28 the radii grow to 1e-14
 // and boxes whose values are that small stay open (monomials of 2^-144 under coefficients of
 // 2^92 were taken for 0 before).
-float screen_tiny(const ivs_system *s, const double *lo, const double *hi) {
+bool float_range(const ivs_system *s, const double *lo, const double *hi, float *scr_tiny) {
     const int n = s->n_vars;
-    double top = 0.0;
+    double m[kMaxVars], top = 0.0;
+    for (int j = 0; j < n; j++) m[j] = std::max({std::fabs(lo[j]), std::fabs(hi[j]), 1.0});
+    bool safe = true;
     for (int i = 0; i < s->n_eqs; i++) {
+        const int nt = s->eq_offsets[i + 1] - s->eq_offsets[i];
         double sum = 0.0;
         for (int t = s->eq_offsets[i]; t < s->eq_offsets[i + 1]; t++) {
-            double b = std::max({std::fabs(s->coef_lo[t]), std::fabs(s->coef_hi ? s->coef_hi[t] : s->coef_lo[t]), 1.0});
+            const double c = std::max(std::fabs(s->coef_lo[t]), std::fabs(s->coef_hi ? s->coef_hi[t] : s->coef_lo[t]));
+            double b = c, p = std::max(c, 1.0);   // magnitude; the same with |c| at least 1
             int g = 0;
             for (int j = 0; j < n; j++) {
                 const int a = s->exps[(size_t)t * n + j];
-                const double m = std::max({std::fabs(lo[j]), std::fabs(hi[j]), 1.0});
                 g += a;
-                for (int q = 0; q < a; q++) b *= m;
+                for (int q = 0; q < a; q++) {
+                    b *= m[j];
+                    p *= m[j];
+                }
             }
-            sum += (g + 1) * b;
+            safe = safe && b * (nt + 1) < 1e30;
+            sum += (g + 1) * p;
         }
         top = std::max(top, sum);
     }
-    return to_float_up((double)kScrTiny + std::ldexp(top, -144));
+    *scr_tiny = to_float_up((double)kScrTiny + std::ldexp(top, -144));
+    return safe;
 }
 
+// F_i and J_ij polynomials of one system appended to the tables.  J_ij = sum over terms t
+// of equation i with a_tj > 0 of [down(c_lo a_tj), up(c_hi a_tj)] x^(a_t - e_j), in term
+// order; its factors keep the variable order of the term.
 void compile_system(HostTables &h, const ivs_system *s, const ivs_options *o) {
     const int n = s->n_vars, m = s->n_eqs;
     SysBuild bld;

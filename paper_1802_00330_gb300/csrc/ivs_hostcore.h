@@ -51,10 +51,9 @@ struct HostTables {
 int validate(const ivs_system *s, const double *lo, const double *hi, const ivs_options *o);
 // appends the system's blob and DevSys (options folded in; shadow off)
 void compile_system(HostTables &h, const ivs_system *s, const ivs_options *o);
-// true when no FP32 shadow intermediate can overflow on this machine
-bool shadow_safe(const ivs_system *s, const double *lo, const double *hi);
-// what float underflow may add to the value of one of the system's polynomials on this machine
-float screen_tiny(const ivs_system *s, const double *lo, const double *hi);
+// true when no FP32 shadow intermediate can overflow on this machine; *scr_tiny: what float underflow
+// may add to the value of one of the system's polynomials there
+bool float_range(const ivs_system *s, const double *lo, const double *hi, float *scr_tiny);
 
 size_t align_up(size_t v, size_t a);
 struct Layout {

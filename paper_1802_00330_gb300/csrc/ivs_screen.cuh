@@ -133,7 +133,7 @@ __device__ __forceinline__ void pow32(float l, float h, float m, int k, float &a
 // ends are real interval arithmetic up to rounding, so the float ends differ from them by at
 // most (operations + input roundings) x 2^-24 x the sum of the terms' magnitudes, plus what
 // products lose below float's normal range: tiny, a bound over the system's initial box
-// (host::screen_tiny).  Magnitudes that underflow themselves are covered by it too.
+// (host::float_range).  Magnitudes that underflow themselves are covered by it too.
 // Terms of up to three factors of degree up to kScrPow read the box's powers (pl, ph: computed
 // once per box, stride 32) and one 16-byte record; the others go through the term table.
 // (With the table alone every term decoded its factors and raised its powers again; with that, the

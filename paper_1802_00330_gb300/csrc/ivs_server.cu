@@ -324,8 +324,8 @@ int ivs_server::step(std::vector<std::pair<uint64_t, ivs_result *>> &finished) {
             region_free(s);
             continue;
         }
-        d.shadow = (rq.opt.prefilter_fp32 && shadow_safe(&sv, rq.lo.data(), rq.hi.data())) ? 1 : 0;
-        d.scr_tiny = screen_tiny(&sv, rq.lo.data(), rq.hi.data());
+        const bool in_range = float_range(&sv, rq.lo.data(), rq.hi.data(), &d.scr_tiny);
+        d.shadow = (rq.opt.prefilter_fp32 && in_range) ? 1 : 0;
         d.blob_off = (int64_t)s * kBlobSlot;
         d.out_base = (int64_t)s * rps;
         d.out_cap = rq.opt.max_results > 0 ? std::min<int64_t>(rq.opt.max_results, rps) : rps;
