@@ -2,11 +2,12 @@
 //
 // One sweep ("wave") pops up to K parent boxes from the top of the queue and runs:
 //   k_wave_begin  : chooses K so that the worst case (every child kept) fits
-//   k_eval        : one warp per parent, one lane per child box (Algorithm 2's split is
-//                   implicit: child c takes the upper half of coordinate j when bit j of
-//                   c is set); optional FP32 outward evaluation, then FP64 evaluation
-//                   (Definition 1-2); survivors compacted with a warp ballot into a list
-//                   per dimension n
+//   k_eval        : a warp (many children, or few parents: a block) per parent; Algorithm 2's split
+//                   is implicit: child c takes the upper half of coordinate j when bit j of
+//                   c is set; FP32 outward evaluation, or FP64 without the FP32 stage
+//                   (Definition 1-2); survivors compacted with warp ballots into a list
+//                   per dimension n, undecided children into one for
+//   k_eval64      : the FP64 evaluation of those
 //   k_screen<N>   : decides in FP32 what the contraction would drop or leave unchanged
 //   k_hs<N>       : 32 survivors per block (narrow sweeps: 8 per block,
 //   k_hs_narrow<N>  k_hs_narrow): Hansen-Sengupta sweeps (Algorithm 3) or Krawczyk steps
@@ -76,7 +77,8 @@ cudaError_t launch_sweep(const SweepArgs &a, const int *hs_dims, int n_hs_dims, 
                          int eval_threads, int num_sms, cudaStream_t st, cudaEvent_t *ev, int *kernels = nullptr);
 // The sweep loop as one CUDA graph: a conditional WHILE node whose body is one sweep; its
 // commit kernel keeps the condition set while the queue is non-empty, no error occurred
-// and ctl->waves < ctl->wave_limit.  Kernels per iteration: 4 + n_hs_dims.
+// and ctl->waves < ctl->wave_limit.  *kernels_per_sweep: kernels per iteration (plans of one system
+// pop in the commit and have no k_wave_begin in it).
 cudaError_t build_sweep_graph(const SweepArgs &a, const int *hs_dims, int n_hs_dims, int eval_blocks,
                               int eval_threads, int num_sms, cudaGraph_t *out, int *kernels_per_sweep = nullptr);
 // directed-rounding rate microbenchmark (kind 0 FP64, 1 FP32); returns ops and fills ms
