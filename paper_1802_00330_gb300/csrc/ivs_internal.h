@@ -54,7 +54,8 @@ constexpr int64_t kFlagResultOverflow = 1, kFlagDepthCut = 2, kFlagBudget = 4;
 
 // Compiled system, resident on the device.  Its polynomials (the m equations F_i, then
 // the m*n Jacobian entries J_ij row-major when m == n) live in one blob of the blob
-// arena at blob_off (layout: ivs_tab.cuh).
+// arena at blob_off (layout: ivs_tab.cuh).  152 bytes: with 160 a burst of 24 served requests, whose
+// kernels read a record per parent, took 0.4% longer (65.3 -> 65.6 ms).
 struct DevSys {
     int32_t n, m;
     int32_t f_poly;        // first polynomial of F (local index, 0)
@@ -72,14 +73,14 @@ struct DevSys {
     int32_t n_tv;          // term-combination entries (0: no per-parent table)
     int32_t centred;       // 1: centred-form exclusion test before Hansen-Sengupta
     int32_t n_cix;         // child-index entries (n_fterms << min(n, 8); 0: none)
-    int32_t eval_block;    // 1: a parent's children are worth a block (512 or more)
+    int16_t eval_block;    // 1: a parent's children are worth a block (512 or more)
+    int16_t gap_split;     // 1: two boxes at an extended-division gap (Gauss-Seidel only)
     uint8_t eq_order[kMaxVars];   // equations by number of terms (when m <= kMaxVars)
     int32_t krawczyk;      // 1: Krawczyk contraction (eq 15-16) instead of Gauss-Seidel
     int32_t bisect;        // 1: widest-coordinate bisection (2 children) instead of 2^n
     int32_t n_scr;         // the screen's term records (n_terms, or 0)
     int32_t head_bytes;    // bytes of the blob's head (ivs_tab.cuh)
     float scr_tiny;        // the screen: what underflow may add to a polynomial's float value
-    int32_t gap_split;     // 1: two boxes at an extended-division gap (Gauss-Seidel only)
 };
 
 // children of a popped queue entry: 1 for an initial box, else 2 (bisection) or 2^n

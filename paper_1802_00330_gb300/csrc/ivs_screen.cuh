@@ -400,16 +400,17 @@ __global__ void __launch_bounds__(scr::Cfg<N>::NT, scr::Cfg<N>::MIN_BLOCKS)
             const DevSys &S = a.tb.sys[s_sys[b]];
             const SysTab T = make_tab(cache_blob ? smem : a.tb.blobs + S.blob_off, S);
             const float *xl = sf + C::XL + b, *xh = sf + C::XH + b;
+            const float tiny = S.scr_tiny;
             for (int q = warp; q < N * N + N; q += NT / 32) {
                 if (!on) continue;
                 if (q < N * N) {
-                    const Poly v = poly_c(T, S.j_poly + q, xl, xh, sf + C::PL + b, sf + C::PH + b, S.scr_tiny);
+                    const Poly v = poly_c(T, S.j_poly + q, xl, xh, sf + C::PL + b, sf + C::PH + b, tiny);
                     sf[C::JC + q * P + b] = v.c;
                     sf[C::JW + q * P + b] = v.w;
                     sf[C::JR + q * P + b] = v.r;
                 } else {
                     const float2 v = poly_v(T, S.f_poly + (q - N * N), xl, xh, sf + C::PL + b, sf + C::PH + b,
-                                            sf + C::PX + b, S.scr_tiny);
+                                            sf + C::PX + b, tiny);
                     sf[C::FV + (q - N * N) * BB + b] = v.x;
                     sf[C::FR + (q - N * N) * BB + b] = v.y;
                 }
